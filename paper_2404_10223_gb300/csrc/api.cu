@@ -356,8 +356,8 @@ struct RotBatch {
   std::vector<std::vector<int>> cap;     // per pair: N + 1 capacities
   std::vector<std::vector<long long>> woff;
   std::vector<long long> work_base;      // doubles, per pair
-  std::vector<long long> scratch_base;   // doubles, per pair (theta + wbuf + qbuf)
-  std::vector<long long> scratch_len;
+  std::vector<long long> scratch_base;   // doubles, per pair (theta, block buffers, exchange area)
+  std::vector<long long> scratch_len, block_len, tiles;
   // device views per pair
   std::vector<double*> work;
   std::vector<int*> dims;
@@ -464,16 +464,30 @@ void run_rotations(tnqe_ctx* c, const std::vector<std::pair<int, int>>& pairs, R
       off[s] = tot;
       tot += (long long)cap[s] * 4 * cap[s + 1];
     }
-    long long th = 16;
+    long long th = 16, blk = 64;
     for (int a = 0; a + 1 < N; ++a) th = std::max(th, 16LL * cap[a] * cap[a + 2]);
     for (int a = 0; a < N; ++a) th = std::max(th, 4LL * cap[a] * cap[a + 1]);   // one site at capacity
+    // The SVD blocks of one gate: a block's rows number at most cap[a] and its columns cap[a + 2], and the
+    // rows (columns) of all blocks add up to 4 times that, so sum m n <= 4 cap[a] cap[a + 2] and
+    // sum (m + n) <= 4 (cap[a] + cap[a + 2]); m is padded to 16 and n to 8 (16 in the digit tiles).
+    long long tiles = 1;
+    for (int a = 0; a + 1 < N; ++a) {
+      const long long cl = cap[a], cr = cap[a + 2], nb = std::min<long long>(QSPACE, 4 * std::min(cl, cr));
+      blk = std::max(blk, 4 * cl * cr + 60 * (cl + cr) + 105 * nb);
+      tiles = std::max(tiles, (4 * cl * cr + 60 * (cl + cr) + 225 * nb) / 256 + 1);
+    }
+    blk = (blk + 63) & ~63LL;
+    th = (th + 63) & ~63LL;
     rb.cap.push_back(cap);
     rb.woff.push_back(off);
     rb.work_base.push_back(work_total);
     work_total += tot;
     rb.scratch_base.push_back(scratch_total);
     rb.scratch_len.push_back(th);
-    scratch_total += 6 * th;
+    rb.block_len.push_back(blk);
+    rb.tiles.push_back(tiles);
+    // theta; eight FP64 block buffers, two FP32; the digit fragments; the exchange area
+    scratch_total += th + 9 * blk + tiles * ROT_TILE_DOUBLES + ROT_XCHG_BYTES / 8;
   }
   // small per-pair arrays: dims (N+1 ints), caps, offsets, sectors, disc, status
   auto al256 = [](size_t x) { return (x + 255) & ~(size_t)255; };
@@ -481,7 +495,8 @@ void run_rotations(tnqe_ctx* c, const std::vector<std::pair<int, int>>& pairs, R
   const size_t per_small = al256(sec_bytes + 2 * 256 + (size_t)(N + 1) * 8 * 2 + (size_t)N * 8 + 64);
   c->rot_work.ensure(sizeof(double) * std::max<long long>(work_total, 1));
   c->rot_scratch.ensure(sizeof(double) * std::max<long long>(scratch_total, 1));
-  c->rot_meta.ensure(sizeof(int) * META_INTS * np);
+  const int cluster = rotate_cluster(np);
+  c->rot_meta.ensure(sizeof(int) * META_INTS * np * cluster);
   c->rot_small.ensure(per_small * np);
   c->rot_desc.ensure(sizeof(RotDesc) * np);
   std::vector<unsigned char> small(per_small * np, 0);
@@ -531,14 +546,22 @@ void run_rotations(tnqe_ctx* c, const std::vector<std::pair<int, int>>& pairs, R
     d.gate_side = pl->d_side;
     double* sb = c->rot_scratch.as<double>() + rb.scratch_base[k];
     const long long th = rb.scratch_len[k];
+    const long long blk = rb.block_len[k];
     d.theta = sb;
+    d.blk_cap = blk;
+    d.tile_cap = rb.tiles[k];
     d.bbuf = sb + th;
-    d.wbuf = sb + 2 * th;
-    d.qbuf = sb + 3 * th;
-    d.tbuf = sb + 4 * th;
-    d.w32 = reinterpret_cast<float*>(sb + 5 * th);
-    d.q32 = d.w32 + th;
-    d.meta = c->rot_meta.as<int>() + META_INTS * k;
+    d.wgbuf = d.bbuf + blk;
+    d.xdbuf = d.wgbuf + blk;
+    d.dgbuf = d.xdbuf + blk;
+    d.wbuf = d.dgbuf + 2 * blk;
+    d.qbuf = d.wbuf + blk;
+    d.tbuf = d.qbuf + blk;
+    d.w32 = reinterpret_cast<float*>(d.tbuf + blk);
+    d.q32 = d.w32 + blk;
+    d.frag = reinterpret_cast<uint4*>(d.tbuf + 2 * blk);
+    d.xchg = d.tbuf + 2 * blk + rb.tiles[k] * ROT_TILE_DOUBLES;
+    d.meta = c->rot_meta.as<int>() + META_INTS * cluster * k;
     d.meta_cap = META_INTS;
     d.discarded = ddisc;
     d.status = dstat;
@@ -567,7 +590,7 @@ void run_rotations(tnqe_ctx* c, const std::vector<std::pair<int, int>>& pairs, R
   }
   upload(c, c->rot_desc.p, descs.data(), sizeof(RotDesc) * np);
   record_event(c, c->pev[0]);
-  CKL(launch_rotate(c->rot_desc.as<RotDesc>(), np, 0, c->stream));
+  CKL(launch_rotate(c->rot_desc.as<RotDesc>(), np, cluster, c->stream));
   c->launches += 1;
   record_event(c, c->pev[1]);
 }

@@ -58,6 +58,8 @@ struct Mpo {
 Mpo build_mpo(const double* h1, const double* eri, int N);
 
 // ----------------------------------------------------------------------------- device descriptors
+constexpr int ROT_XCHG_BYTES = 20480;
+constexpr int ROT_TILE_DOUBLES = 2 * 7 * 64;   // digit fragments of a 16 x 16 tile and its transpose
 struct RotDesc {
   int N, chi_rot, ngates, neg_site, renorm, max_sweeps;
   int pad_out, pad_;              // pad_out: leave every site as [cap_l][4][cap_r], zero-filled
@@ -75,13 +77,20 @@ struct RotDesc {
   const int* gate_site;
   const int* gate_side;
   double* theta;                  // scratch: two-site tensor
-  double* bbuf;                   // SVD blocks (scaled copies of the gated two-site blocks)
+  long long blk_cap;              // doubles of each block buffer below
+  long long tile_cap;             // 16 x 16 tiles of the digit fragments
+  double* bbuf;                   // SVD blocks B, column-major
+  double* wgbuf;                  // B X (double-floats)
+  double* xdbuf;                  // X (double-floats)
+  double* dgbuf;                  // digits of either (2 blk_cap)
+  uint4* frag;                    // digit fragments of B and B^T (2 x 7 x 32 per tile)
   double* wbuf;                   // B V per block
   double* qbuf;                   // V per block
   double* tbuf;                   // n x n temporaries per block
   float* w32;                     // FP32 working copy of each block
-  float* q32;                     // FP32 rotations of each block
-  int* meta;                      // scratch ints
+  float* q32;                     // FP32 singular vectors of each block
+  void* xchg;                     // exchange area of the pair's CTAs (ROT_XCHG_BYTES)
+  int* meta;                      // scratch ints, meta_cap for each CTA of the pair
   long long meta_cap;
   double* discarded;
   int* status;
@@ -201,7 +210,8 @@ constexpr int STATUS_NOCONV = 1;
 constexpr int STATUS_OVERFLOW = 2;
 
 // kernel launchers (kernels_*.cu); return cudaError_t as int
-int launch_rotate(const RotDesc* d_descs, int npairs, int smem_bytes, void* stream);
+int rotate_cluster(int npairs);      // CTAs per pair the rotation of npairs pairs is launched with
+int launch_rotate(const RotDesc* d_descs, int npairs, int cluster, void* stream);
 int launch_gemm_f64(const GemmDesc* d_descs, const long long* d_tile_prefix, int nprob,
                     long long total_tiles, void* stream);
 int launch_spmm_f64(const SpmmDesc* d_descs, const long long* d_row_prefix, int nprob,

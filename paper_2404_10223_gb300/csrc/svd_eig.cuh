@@ -1,0 +1,1173 @@
+// Truncated SVD of one charge block by an FP32 eigendecomposition and a
+// refinement of the kept singular vectors alone.
+//
+// A gate keeps about a quarter of its singular triplets (chi of up to 4 chi),
+// and only the kept ones are needed to full precision.  So, for a block B
+// (m x n, n <= m):
+//   1. eig_start:  G = B^T B to FP32, Householder tridiagonalisation, all
+//      eigenvalues by multisection (Sturm counts), eigenvectors of the
+//      tridiagonal matrix by inverse iteration (LU with partial pivoting,
+//      two steps), back-transformation, Newton-Schulz steps until the vectors
+//      X are orthonormal to FP32.  About 3 n^3 multiply-adds with one team
+//      barrier per Householder step, against 7 sweeps of 6 n^3 for one-sided
+//      Jacobi in FP32.
+//   2. (the caller decides from the eigenvalues, with error bounds, which
+//      columns can be kept at all)
+//   3. eig_refine: for the kept columns x_k alone
+//        w = B x, lambda = |w|^2, r = B^T w - lambda x,
+//      and the first-order correction with all FP32 vectors X as the basis,
+//        x <- x + X t,  t_i = X_i . r / (lambda - lambda_i),  t_k = (1 - |x|^2) / 2
+//      (Ogita and Aishima, Japan J. Indust. Appl. Math. 35 (2018) 1007, with the
+//      residual formed before the projection, so that the products with X and
+//      the update only need FP32).  It converges quadratically: on the gates of
+//      N = 14, chi = 128 states |t| is at most 1e-4, then 1e-8, then at rounding
+//      level, so two corrections.
+// Whatever this cannot do (a kept singular value below 5e-3 of the block's
+// largest one, a cluster that leaves X dependent, a correction that does not
+// shrink) is reported, and the caller takes the one-sided Jacobi SVD.
+//
+// The products with B run on the tensor cores with operands cut into 8-bit signed
+// digits (Ozaki, Ogita, Oishi, Rump, Numer. Algorithms 59 (2012) 95): every digit is
+// an exact BF16 number, a digit product is at most 2^14 and the sums of one order are
+// integers below 2^24, so FP32 accumulation is exact, and seven digits (resolution
+// 2^-54 of the block's largest entry) with the 28 products of order up to 8 carry the
+// accuracy of double-float arithmetic (48 bits) or better.  A multiply-add costs 28/2048
+// of a warp-wide mma against 12 FP32 instructions in double-float and 64 issue cycles
+// in FP64 (GB300's FP64 rate is 1/64 of its FP32 rate).  mma.sync and not tcgen05: the
+// blocks are 10 to 80 wide and eight to thirty columns are kept, far below a tcgen05
+// tile, and the operands of a warp come straight from L2 in fragment order.
+#pragma once
+#include <cuda_runtime.h>
+
+#include "df.cuh"
+
+namespace tnqe {
+namespace {
+
+constexpr int EIG_NE = 5;                          // lanes' share of a row: n <= 32 EIG_NE
+constexpr int EIG_MAXN = 32 * EIG_NE;
+constexpr float EIG_MIN_LAMBDA = 3e-5f;            // kept lambda over the block's largest: sigma ratio 5.5e-3
+constexpr int EIG_TC = 8;                          // kept columns per task (an mma's n)
+constexpr int EIG_DIG = 7;                         // digits of an operand
+constexpr int EIG_WEXP = 4;                        // |w| < 2^(1 + EIG_WEXP): 2 sqrt(256)
+
+__device__ __forceinline__ float warp_sum_f(float v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+__device__ __forceinline__ float warp_max_f(float v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+// Row stride of the n x n FP32 arrays: a multiple of 4 (16-byte rows) and 4 mod 8, so
+// that 16-byte accesses of eight consecutive rows fall into distinct banks.
+__host__ __device__ __forceinline__ int eig_ld(int n) {
+  const int l = (n + 3) & ~3;
+  return (l & 7) == 4 ? l : l + 4;
+}
+__host__ __device__ __forceinline__ int eig_kp(int k) { return (k + EIG_TC - 1) & ~(EIG_TC - 1); }
+__host__ __device__ __forceinline__ int pad16(int n) { return (n + 15) & ~15; }
+// floats of the small vectors of eig_start (V: 2 ld, W: ld, P: 2 ld, d, e, tau, lam, scale, a dummy row)
+__host__ __device__ __forceinline__ int eig_vec_floats(int n) { return 11 * eig_ld(n) + 32; }
+// Tells the compiler that a generic pointer points to shared memory.
+#define EIG_SHARED(p) __builtin_assume(__isShared(p))
+
+// s + e accumulates a b (double-floats): the compensated dot product of Ogita, Rump
+// and Oishi (SIAM J. Sci. Comput. 26 (2005) 1955), as accurate as twice FP32.
+__device__ __forceinline__ void dot2_step(float2 a, float2 b, float& s, float& e) {
+  const float p = __fmul_rn(a.x, b.x);
+  float pe = __fmaf_rn(a.x, b.x, -p);
+  float t, u;
+  dfa::two_sum(s, p, t, u);
+  s = t;
+  pe = __fmaf_rn(a.x, b.y, pe);
+  pe = __fmaf_rn(a.y, b.x, pe);
+  e = __fadd_rn(e, __fadd_rn(u, pe));
+}
+__device__ __forceinline__ float2 df_pair(float s, float e) {
+  float2 r;
+  dfa::two_sum(s, e, r.x, r.y);
+  return r;
+}
+
+// Uniform in [-1, 1] from a pair of indices (a start vector only has to be generic).
+__device__ __forceinline__ float eig_noise(unsigned i, unsigned u) {
+  unsigned h = i * 0x9E3779B1u ^ (u + 0x7F4A7C15u) * 0x85EBCA77u;
+  h ^= h >> 15;
+  h *= 0x2C1B3C6Du;
+  h ^= h >> 12;
+  h *= 0x297A2D39u;
+  h ^= h >> 15;
+  return (float)(int)h * 4.656612873e-10f;
+}
+
+// ----------------------------------------------------------------------------- digits and mma fragments
+// A value v, |v| < 2, is the integer I = v 2^54 and I = sum_{s=1..7} d_s 2^(8 (7 - s)), d_s in
+// [-128, 128]: v = sum d_s 2^(2 - 8 s).
+__device__ __forceinline__ long long fix_float(float x, int ex) {   // x 2^(54 - ex), |x| < 2^(1 + ex)
+  const unsigned b = (unsigned)__float_as_int(x);
+  const int e = (int)((b >> 23) & 255);
+  const long long m = e ? (long long)((b & 0x7fffffu) | 0x800000u) : 0;
+  const int sh = e - 96 - ex;
+  const long long v = sh >= 0 ? m << min(sh, 40) : (sh > -25 ? m >> -sh : 0);
+  return (b >> 31) ? -v : v;
+}
+__device__ __forceinline__ long long fix_df(float2 v, int ex) { return fix_float(v.x, ex) + fix_float(v.y, ex); }
+// x / 2^ex 2^54 of a double, |x| < 2^(1 + ex)
+__device__ __forceinline__ long long fix_double(double x, int ex) {
+  const long long b = __double_as_longlong(x);
+  const int e = (int)((b >> 52) & 2047);
+  const long long m = e ? ((b & 0xfffffffffffffll) | 0x10000000000000ll) : 0;
+  const int sh = e - 1023 - ex + 2;
+  const long long v = sh >= 0 ? m << min(sh, 10) : (sh > -54 ? m >> -sh : 0);
+  return b < 0 ? -v : v;
+}
+// the digits of a pair of integers as BF16 pairs (first in the low half)
+__device__ __forceinline__ void digits_pair(long long a, long long b, unsigned (&w)[EIG_DIG]) {
+  const long long bias = 0x808080808080ll;
+  a += bias;
+  b += bias;
+  const float ta = __int_as_float(0x4B400000 + (int)(a >> 48)) - 12582912.f;
+  const float tb = __int_as_float(0x4B400000 + (int)(b >> 48)) - 12582912.f;
+  w[0] = __byte_perm((unsigned)__float_as_int(ta), (unsigned)__float_as_int(tb), 0x7632);
+  const unsigned al = (unsigned)a, ah = (unsigned)((unsigned long long)a >> 32);
+  const unsigned bl = (unsigned)b, bh = (unsigned)((unsigned long long)b >> 32);
+#pragma unroll
+  for (int s = 1; s < EIG_DIG; ++s) {
+    const int by = EIG_DIG - 1 - s;                // byte 5 .. 0
+    const unsigned sel = 0x7440u | (by & 3);       // byte, 0, 0, 0x4B
+    const float fa = __int_as_float((int)__byte_perm(by > 3 ? ah : al, 0x4B000000u, sel)) - 8388736.f;
+    const float fb = __int_as_float((int)__byte_perm(by > 3 ? bh : bl, 0x4B000000u, sel)) - 8388736.f;
+    w[s] = __byte_perm((unsigned)__float_as_int(fa), (unsigned)__float_as_int(fb), 0x7632);
+  }
+}
+__device__ __forceinline__ unsigned transpose8x8(unsigned x) {
+  unsigned r;
+  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(x));
+  return r;
+}
+__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint4& a, const uint2& b) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y));
+}
+
+// A-operand fragments of B (rows of B) in A and of B^T in At, tile by tile: the 16 x 16 tile
+// (it, kt) of a matrix with KT column tiles has its EIG_DIG digits at ((it KT + kt) EIG_DIG + s) 32
+// + lane.  raw: B column-major (m x n), |entries| < 2^(1 + ex).  A warp takes a tile of
+// B; its transpose comes from the registers (movmatrix).
+template <class Team>
+__device__ __noinline__ void eig_digits(const Team tm, const double* raw, int m, int n, int ex, uint4* A, uint4* At) {
+  const int lane = threadIdx.x & 31, warp = tm.rank() >> 5, nw = tm.size() >> 5;
+  const int mt = pad16(m) >> 4, nt = pad16(n) >> 4, g = lane >> 2, t2 = 2 * (lane & 3);
+  for (int t = warp; t < mt * nt; t += nw) {
+    const int it = t % mt, kt = t / mt;
+    long long v[4][2];                             // registers (rows g, g + 8) x (columns t2, t2 + 8), pairs along the row
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int r = 16 * it + g + 8 * (q & 1), c = 16 * kt + t2 + 8 * (q >> 1) + h;
+        v[q][h] = (r < m && c < n) ? fix_double(raw[(size_t)c * m + r], ex) : 0;
+      }
+    unsigned w[4][EIG_DIG];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) digits_pair(v[q][0], v[q][1], w[q]);
+    uint4* a = A + (size_t)(it * nt + kt) * EIG_DIG * 32 + lane;
+    uint4* b = At + (size_t)(kt * mt + it) * EIG_DIG * 32 + lane;
+#pragma unroll
+    for (int s = 0; s < EIG_DIG; ++s) {
+      a[s * 32] = make_uint4(w[0][s], w[1][s], w[2][s], w[3][s]);
+      b[s * 32] = make_uint4(transpose8x8(w[0][s]), transpose8x8(w[2][s]), transpose8x8(w[1][s]), transpose8x8(w[3][s]));
+    }
+  }
+  tm.sync();
+}
+
+// B-operand fragments of the columns k = 0..kp-1 of V (column k at k ldv, double-floats, |entries| <
+// 2^(1 + ex), length K padded with zeros to a multiple of 16): the 16 x 8 tile (kt, jt) has its digits
+// at ((kt JT + jt) ND + s) 32 + lane.
+template <int ND, class Team>
+__device__ __noinline__ void eig_digits_cols(const Team tm, const float2* V, int ldv, int K, int kp, int ex, uint2* D) {
+  const int lane = threadIdx.x & 31, warp = tm.rank() >> 5, nw = tm.size() >> 5;
+  const int kt = pad16(K) >> 4, jt = kp >> 3, g = lane >> 2, t2 = 2 * (lane & 3);
+  for (int t = warp; t < kt * jt; t += nw) {
+    const int k = t / jt, j = t % jt;
+    const float4* p = reinterpret_cast<const float4*>(V + (size_t)(8 * j + g) * ldv + 16 * k + t2);
+    const float4 lo = p[0], hi = p[4];
+    unsigned a[EIG_DIG], b[EIG_DIG];
+    digits_pair(fix_df(make_float2(lo.x, lo.y), ex), fix_df(make_float2(lo.z, lo.w), ex), a);
+    digits_pair(fix_df(make_float2(hi.x, hi.y), ex), fix_df(make_float2(hi.z, hi.w), ex), b);
+    uint2* d = D + (size_t)t * ND * 32 + lane;
+#pragma unroll
+    for (int s = 0; s < ND; ++s) d[s * 32] = make_uint2(a[s], b[s]);
+  }
+  tm.sync();
+}
+
+// One 16 x 8 tile of the product: NA digits of the first operand (tile row `it`, KT tiles), NB of the
+// second (tile column j of JT), products of order up to NS.  acc[o] holds the sums of order
+// o + 2 in units of 2^(4 - 8 (o + 2)).
+template <int NA, int NB, int NS>
+__device__ __forceinline__ void mma_tile(const uint4* A, const uint2* D, int it, int j, int KT, int JT, int lane,
+                                         float (&acc)[NS - 1][4]) {
+#pragma unroll
+  for (int o = 0; o < NS - 1; ++o)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[o][q] = 0.f;
+  const uint4* ap = A + (size_t)it * KT * EIG_DIG * 32 + lane;
+  uint4 an[NA];
+#pragma unroll
+  for (int s = 0; s < NA; ++s) an[s] = ap[s * 32];
+  for (int k = 0; k < KT; ++k) {
+    uint4 a[NA];
+    uint2 b[NB];
+#pragma unroll
+    for (int s = 0; s < NA; ++s) a[s] = an[s];
+    const uint2* bp = D + (size_t)(k * JT + j) * NB * 32 + lane;
+#pragma unroll
+    for (int s = 0; s < NB; ++s) b[s] = bp[s * 32];
+    if (k + 1 < KT) {
+      ap += EIG_DIG * 32;
+#pragma unroll
+      for (int s = 0; s < NA; ++s) an[s] = ap[s * 32];
+    }
+#pragma unroll
+    for (int i = 0; i < NA; ++i)
+#pragma unroll
+      for (int s = 0; s < NB; ++s)
+        if (i + s + 2 <= NS) mma_bf16(acc[i + s], a[i], b[s]);
+  }
+}
+// The sums of all orders as a double-float, times 2^e (smallest order first).
+template <int NS>
+__device__ __forceinline__ float2 mma_value(const float (&acc)[NS - 1][4], int q, int e) {
+  float2 v = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int o = NS - 2; o >= 0; --o) {
+    const float x = acc[o][q] * __int_as_float((127 + 4 - 8 * (o + 2)) << 23);
+    float s, r;
+    dfa::two_sum(x, v.x, s, r);
+    v = dfa::fast_two_sum(s, __fadd_rn(r, v.y));
+  }
+  const float f = __int_as_float((127 + e) << 23);
+  return make_float2(v.x * f, v.y * f);
+}
+
+// ----------------------------------------------------------------------------- Gram matrix
+// S (n x n, row stride ld, both triangles, pad columns zero) = B^T B to FP32: three digits, the six
+// products of order up to 4.  The fragments of B^T serve as both operands.
+template <class Team>
+__device__ __noinline__ void eig_gram(const Team tm, const uint4* At, int m, int n, float* S, int ld) {
+  EIG_SHARED(S);
+  const int tr = tm.rank(), ts = tm.size(), lane = threadIdx.x & 31, warp = tr >> 5, nw = ts >> 5;
+  const int mt = pad16(m) >> 4, nt = pad16(n) >> 4, g = lane >> 2, t2 = 2 * (lane & 3);
+  for (int x = tr; x < n * (ld - n); x += ts) S[(x / (ld - n)) * ld + n + x % (ld - n)] = 0.f;
+  for (int t = warp; t < nt * 2 * nt; t += nw) {
+    const int it = t / (2 * nt), j8 = t % (2 * nt), jt = j8 >> 1;
+    if (jt < it || 8 * j8 >= n) continue;
+    float acc[3][4];
+#pragma unroll
+    for (int o = 0; o < 3; ++o)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[o][q] = 0.f;
+    const uint4* ap = At + (size_t)it * mt * EIG_DIG * 32 + lane;
+    const uint4* bp = At + (size_t)jt * mt * EIG_DIG * 32 + lane;
+#pragma unroll 2
+    for (int k = 0; k < mt; ++k) {
+      uint4 a[3];
+      uint2 b[3];
+#pragma unroll
+      for (int s = 0; s < 3; ++s) {
+        a[s] = ap[(k * EIG_DIG + s) * 32];
+        const uint4 v = bp[(k * EIG_DIG + s) * 32];
+        b[s] = (j8 & 1) ? make_uint2(v.y, v.w) : make_uint2(v.x, v.z);
+      }
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int s = 0; s + i < 3; ++s) mma_bf16(acc[i + s], a[i], b[s]);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = 16 * it + g + 8 * (q >> 1), j = 8 * j8 + t2 + (q & 1);
+      if (i < n && j < n) {
+        const float v = fmaf(acc[0][q], 0x1p-12f, fmaf(acc[1][q], 0x1p-20f, acc[2][q] * 0x1p-28f));
+        S[i * ld + j] = v;
+        if (jt > it) S[j * ld + i] = v;
+      }
+    }
+  }
+  tm.sync();
+}
+
+// ----------------------------------------------------------------------------- tridiagonalisation
+// Householder reduction of the symmetric A (row stride ld): diagonal d, off-diagonal
+// e, reflectors I - tau v v^T with v left in row j of A (zero up to column j).
+//
+// Latency bound: n - 2 dependent steps, so a step has one team barrier and one
+// reduction.  The rows of the trailing matrix belong to 8-lane groups; a group applies
+// the last rank-2 update to its rows and multiplies them with the new reflector in one
+// pass.  Every warp forms the reflector of row t by itself, from the row in memory,
+// the products p = tau A v of the last step and the last reflector v (v_t = 1):
+//   w = p - K v, K = tau p.v / 2,   row t of A - v w^T - w v^T  =  u + kappa v,
+//   u = a - p, kappa = 2 K - p_t,
+// so that K and the norm of the row come from sums over p, u and v that do not wait
+// for one another (where they cancel, the norm is summed again).  V (two, by parity),
+// W and P (two) hold v, w, p; all warps write the same values into V and W.
+template <int NE, class Team>
+__device__ __noinline__ void eig_tridiag_ne(const Team tm, float* A, int n, int ld, float* V, float* W, float* P, float* d,
+                                            float* e, float* tau, float* dummy) {
+  // 32-bit offsets into the pool: a pointer select per row would cost 64-bit arithmetic
+  extern __shared__ float4 rot_pool[];
+  float* const S = reinterpret_cast<float*>(rot_pool);
+  const int Vo = (int)(V - S), Wo = (int)(W - S), Ao = (int)(A - S), Do = (int)(dummy - S);
+  A = S + Ao;
+  V = S + Vo;
+  W = S + Wo;
+  P = S + (int)(P - S);
+  d = S + (int)(d - S);
+  e = S + (int)(e - S);
+  tau = S + (int)(tau - S);
+  dummy = S + Do;
+  const int tr = tm.rank(), ts = tm.size();
+  const int lane = threadIdx.x & 31, grp = tr >> 3, ngrp = ts >> 3, gl = tr & 7;
+  const unsigned gmask = 0xffu << ((lane >> 3) * 8);
+  const bool first = tr < 32;
+  for (int c = tr; c < ld; c += ts) {
+    V[c] = 0.f;
+    V[ld + c] = 0.f;
+    W[c] = 0.f;
+    P[c] = 0.f;
+    P[ld + c] = 0.f;
+    dummy[c] = 0.f;                                // stays finite: its products meet zeros
+  }
+  tm.sync();
+  float v[NE];
+  float tl = 0.f;                                  // tau of the last reflector
+  int rfirst = grp;                                // the group's first row of the trailing matrix
+#pragma unroll
+  for (int q = 0; q < NE; ++q) v[q] = 0.f;
+  for (int t = 0; t + 1 < n; ++t) {
+    float* Vc = V + (t & 1) * ld;                  // this step's reflector
+    const float* Vp = V + ((t & 1) ^ 1) * ld;      // the last one
+    float* Pc = P + (t & 1) * ld;
+    const float* Pp = P + ((t & 1) ^ 1) * ld;
+    const float* Ar = A + t * ld;
+    const float pt = Pp[t], at = Ar[t];
+    const float an = Ar[t + 1], pn = Pp[t + 1], vnx = Vp[t + 1];
+    float p[NE], u[NE];
+    float s1 = 0.f, s2 = 0.f, s3 = 0.f, s4 = 0.f;
+#pragma unroll
+    for (int q = 0; q < NE; ++q) {
+      const int c = lane + 32 * q;
+      const bool in = c >= t && c < n;
+      p[q] = in ? Pp[c] : 0.f;
+      u[q] = in ? Ar[c] - p[q] : 0.f;
+      s1 = fmaf(p[q], v[q], s1);
+      if (c > t + 1) {
+        s2 = fmaf(u[q], u[q], s2);
+        s3 = fmaf(u[q], v[q], s3);
+        s4 = fmaf(v[q], v[q], s4);
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+      s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+      s3 += __shfl_xor_sync(0xffffffffu, s3, o);
+      s4 += __shfl_xor_sync(0xffffffffu, s4, o);
+    }
+    const float K = 0.5f * tl * s1, kap = 2.f * K - pt;
+    const float x0 = fmaf(kap, vnx, an - pn);
+    if (t + 2 == n) {                              // the last 2 x 2 block needs no reflector
+      if (first && lane == 0) {
+        const int c = n - 1;
+        const float vl = Vp[c], wl = fmaf(-K, vl, Pp[c]);
+        d[t] = at - pt + kap;
+        e[t] = x0;
+        d[c] = A[c * ld + c] - 2.f * vl * wl;
+      }
+      break;
+    }
+    float x[NE];
+#pragma unroll
+    for (int q = 0; q < NE; ++q) x[q] = fmaf(kap, v[q], u[q]);
+    const float big = fmaf(kap * kap, s4, s2);
+    s2 = fmaf(kap, fmaf(kap, s4, 2.f * s3), s2);
+    if (s2 < 0.02f * big) {                        // the sums cancelled
+      s2 = 0.f;
+#pragma unroll
+      for (int q = 0; q < NE; ++q)
+        if (lane + 32 * q > t + 1) s2 = fmaf(x[q], x[q], s2);
+      s2 = warp_sum_f(s2);
+    }
+    float tj = 0.f, beta = x0, inv = 0.f;
+    if (s2 > 1e-30f) {
+      const float h2 = fmaf(x0, x0, s2), ri = rsqrtf(h2), h = h2 * ri;
+      beta = -copysignf(h, x0);
+      tj = fmaf(fabsf(x0), ri, 1.f);
+      inv = copysignf(__fdividef(1.f, fabsf(x0) + h), x0);
+    }
+#pragma unroll
+    for (int q = 0; q < NE; ++q) {
+      const int c = lane + 32 * q;
+      const float w = fmaf(-K, v[q], p[q]);
+      v[q] = (c == t + 1) ? 1.f : ((c > t + 1) ? x[q] * inv : 0.f);
+      if (c < ld) {
+        W[c] = w;
+        Vc[c] = v[q];
+      }
+    }
+    __syncwarp();
+    // rows t + 1.. of the trailing matrix: the last update, and the product with the
+    // reflector, four rows at a time without branches (what lies outside goes to a dummy row)
+    const int c0 = (t + 1) & ~3;
+    if (rfirst < t + 1) rfirst += ngrp;
+    for (int r = rfirst; r < n; r += 4 * ngrp) {
+      float acc[4], vr[4], wr[4];
+      int R[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int ri = r + i * ngrp, rc = min(ri, n - 1);
+        vr[i] = Vp[rc];
+        wr[i] = W[rc];
+        R[i] = ri < n ? Ao + ri * ld : Do;
+        acc[i] = 0.f;
+      }
+      for (int cb = c0; cb < ld; cb += 32) {
+        const bool in = cb + 4 * gl < ld;
+        const int c = in ? cb + 4 * gl : 0;
+        const float4 vp = *reinterpret_cast<const float4*>(Vp + c), wp = *reinterpret_cast<const float4*>(W + c);
+        float4 vc = *reinterpret_cast<const float4*>(Vc + c);
+        float4 a[4];
+        int to[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          to[i] = in ? R[i] + c : Do;
+          a[i] = *reinterpret_cast<const float4*>(S + to[i]);
+        }
+        if (!in) vc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          a[i].x = fmaf(-vr[i], wp.x, fmaf(-wr[i], vp.x, a[i].x));
+          a[i].y = fmaf(-vr[i], wp.y, fmaf(-wr[i], vp.y, a[i].y));
+          a[i].z = fmaf(-vr[i], wp.z, fmaf(-wr[i], vp.z, a[i].z));
+          a[i].w = fmaf(-vr[i], wp.w, fmaf(-wr[i], vp.w, a[i].w));
+          *reinterpret_cast<float4*>(S + to[i]) = a[i];
+          acc[i] = fmaf(a[i].x, vc.x, fmaf(a[i].y, vc.y, fmaf(a[i].z, vc.z, fmaf(a[i].w, vc.w, acc[i]))));
+        }
+      }
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[i] += __shfl_xor_sync(gmask, acc[i], o);
+      // lane i of the group stores the product of row i
+      const float mine = gl == 0 ? acc[0] : (gl == 1 ? acc[1] : (gl == 2 ? acc[2] : acc[3]));
+      if (gl < 4 && r + gl * ngrp < n) Pc[r + gl * ngrp] = tj * mine;
+    }
+    tm.sync();
+    if (first) {                                   // no other warp reads row t any more
+#pragma unroll
+      for (int q = 0; q < NE; ++q)
+        if (lane + 32 * q < ld) A[t * ld + lane + 32 * q] = v[q];
+      if (lane == 0) {
+        d[t] = at - pt + kap;
+        e[t] = beta;
+        tau[t] = tj;
+      }
+    }
+    tl = tj;
+  }
+  if (n == 1 && tr == 0) d[0] = A[0];
+  tm.sync();
+}
+// More than four warps (eight from n = 97 on) only add redundant work to the steps.
+template <class Team>
+__device__ void eig_tridiag(const Team& tm, float* A, int n, int ld, float* V, float* W, float* P, float* d, float* e,
+                            float* tau, float* dummy) {
+  const auto sub = tm.part(n <= 96 ? 128 : 256);
+  if (sub.rank() < sub.size()) {
+    if (n <= 32) eig_tridiag_ne<1>(sub, A, n, ld, V, W, P, d, e, tau, dummy);
+    else if (n <= 64) eig_tridiag_ne<2>(sub, A, n, ld, V, W, P, d, e, tau, dummy);
+    else if (n <= 96) eig_tridiag_ne<3>(sub, A, n, ld, V, W, P, d, e, tau, dummy);
+    else eig_tridiag_ne<EIG_NE>(sub, A, n, ld, V, W, P, d, e, tau, dummy);
+  }
+  tm.sync();
+}
+
+// ----------------------------------------------------------------------------- eigenvalues
+// All eigenvalues of the tridiagonal (d, e), descending in lam, by multisection: two
+// lanes per eigenvalue split its interval in three, fourteen times.  d and e are scaled
+// in place by the returned 1 / norm (the eigenvalues too).  The Sturm sequence is the
+// division-free recurrence p_i = (d_i - x) p_{i-1} - e_{i-1}^2 p_{i-2} (two FMAs per
+// step; a reciprocal per step would be bound by 16 lanes per clock and SM), rescaled
+// every four steps by the exponent of the values four steps before, which keeps the
+// rescaling off the dependent chain; the signs are shifted into a word and counted 32
+// at a time.  de holds the pairs (d_i, e_{i-1}^2).
+template <class Team>
+__device__ __noinline__ float eig_values(const Team tm, float* d, float* e, int n, int ld, float2* de, float* lam) {
+  EIG_SHARED(d);
+  EIG_SHARED(e);
+  EIG_SHARED(de);
+  EIG_SHARED(lam);
+  const int tr = tm.rank(), ts = tm.size(), lane = threadIdx.x & 31;
+  float nm = 0.f;                                  // Gershgorin bound, the same in every warp
+  for (int c = lane; c < n; c += 32)
+    nm = fmaxf(nm, fabsf(d[c]) + (c > 0 ? fabsf(e[c - 1]) : 0.f) + (c + 1 < n ? fabsf(e[c]) : 0.f));
+  nm = warp_max_f(nm);
+  const float sc = nm > 1e-30f ? __fdividef(1.f, nm) : 1.f;
+  tm.sync();
+  for (int c = tr; c < ld; c += ts) {
+    const float ep = (c > 0 && c < n ? e[c - 1] : 0.f) * sc;
+    // pad rows never change a sign: p_i = (2 - x) p_{i-1}
+    de[c] = make_float2(c < n ? d[c] * sc : 2.f, c < n ? fmaxf(ep * ep, 1e-18f) : 0.f);
+  }
+  tm.sync();
+  for (int c = tr; c < ld; c += ts) {
+    d[c] = c < n ? d[c] * sc : 0.f;
+    e[c] = c + 1 < n ? e[c] * sc : 0.f;
+  }
+  const int sub = tr >> 1, nsub = ts >> 1, sl = tr & 1;
+  const unsigned smask = 3u << (lane & 30);
+  const float4* de4 = reinterpret_cast<const float4*>(de);
+  for (int t0 = sub; t0 < n; t0 += nsub) {
+    float lo = -1e-5f, wd = 1.0002f;               // the interval: lo, width
+    for (int pass = 0; pass < 14; ++pass) {
+      const float st = wd * 0.333333343f, x = fmaf((float)(sl + 1), st, lo);
+      float p = 0.f, q = 1.f;                      // p_{i-2}, p_{i-1}
+      unsigned bits = 0, last = 0, cnt = 0;
+      float4 ga = de4[0], gb = de4[1];
+      for (int i = 0; i < n; i += 4) {
+        const float4 ha = ga, hb = gb;
+        if (i + 4 < ld) {
+          ga = de4[(i >> 1) + 2];
+          gb = de4[(i >> 1) + 3];
+        }
+        const int ex = (__float_as_int(fmaxf(fabsf(p), fabsf(q))) >> 23) & 255;
+        const float f = __int_as_float((ex > 40 ? 294 - ex : 254) << 23);     // towards 2^40
+        const float dd[4] = {ha.x, ha.z, hb.x, hb.z}, ee[4] = {ha.y, ha.w, hb.y, hb.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const float r = fmaf(dd[u] - x, q, -(ee[u] * p));
+          bits = __funnelshift_l((unsigned)__float_as_int(r), bits, 1);
+          p = q;
+          q = r;
+        }
+        p *= f;
+        q *= f;
+        if ((i & 31) == 28 || i + 4 >= n) {        // up to 32 signs: their changes, the first against the last word's
+          const int have = (i & 31) + 4;
+          const unsigned al = bits << (32 - have);
+          cnt += __popc((al ^ ((al >> 1) | (last << 31))) & (0xffffffffu << (32 - have)));
+          last = bits & 1u;
+        }
+      }
+      // cnt = eigenvalues below x: the points with at most t0 of them lie below eigenvalue t0 (ascending)
+      const int below = cnt <= (unsigned)t0 ? 1 : 0;
+      const int np = below + __shfl_xor_sync(smask, below, 1);
+      lo = fmaf((float)np, st, lo);
+      wd = st;
+    }
+    if (sl == 0) lam[n - 1 - t0] = fmaf(0.5f, wd, lo);
+  }
+  tm.sync();
+  return sc;
+}
+
+// ----------------------------------------------------------------------------- eigenvectors of the tridiagonal
+// One thread per vector: LU with partial pivoting of T - lam, then two steps of inverse
+// iteration; the first starts from a generic right-hand side after the forward
+// elimination, so it is a back substitution alone.  X[u * ld + i] is component i of
+// vector u; S and M (n x n, row stride n, global memory) keep the pivots and the
+// multipliers, read eight rows ahead of their use.  A row swap at step i shows as
+// |pivot_i| < |e_i|.  inorm[u] gets 1 / |vector u|.
+template <bool XS, class Team>
+__device__ __noinline__ void eig_vectors(const Team tm, const float* d, const float* e, const float* lam, int n,
+                                         float* X, int ld, float* S, float* M, float* inorm) {
+  EIG_SHARED(d);
+  EIG_SHARED(e);
+  EIG_SHARED(lam);
+  EIG_SHARED(inorm);
+  if (XS) EIG_SHARED(X);
+  const int tr = tm.rank(), ts = tm.size();
+  constexpr float TINY = 3e-8f;                    // of |T| = 1
+  constexpr int AH = 8;
+  for (int u = tr; u < n; u += ts) {
+    const float x = lam[u];
+    float* Xu = X + u * ld;
+    float a = d[0] - x, b = e[0];
+    for (int i = 0; i + 1 < n; i += 4) {
+      // rows i .. i + 3: d_{i+1..i+4}, e_{i..i+4} (zero beyond the end)
+      const float4 e4 = *reinterpret_cast<const float4*>(e + i), d4 = *reinterpret_cast<const float4*>(d + i);
+      const float el = i + 4 < ld ? e[i + 4] : 0.f, dl = i + 4 < ld ? d[i + 4] : 0.f;
+      const float ev[5] = {e4.x, e4.y, e4.z, e4.w, el}, dv[4] = {d4.y, d4.z, d4.w, dl};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (i + k + 1 < n) {
+          const float ei = ev[k], en = ev[k + 1], dn = dv[k] - x;
+          const bool swp = fabsf(a) < fabsf(ei);
+          if (!swp && fabsf(a) < TINY) a = copysignf(TINY, a);
+          const float mlt = __fdividef(swp ? a : ei, swp ? ei : a);
+          S[(i + k) * n + u] = a;
+          M[(i + k) * n + u] = mlt;
+          a = fmaf(-mlt, swp ? dn : b, swp ? b : dn);
+          b = swp ? -mlt * en : en;
+        }
+      }
+    }
+    if (fabsf(a) < TINY) a = copysignf(TINY, a);
+    const float ial = __fdividef(1.f, a);
+    float f = 1.f;
+    for (int it = 0; it < 2; ++it) {
+      float r = 0.f;
+      if (it) {                                    // forward elimination of the first vector
+        r = Xu[0] * f;
+        for (int i0 = 0; i0 + 1 < n; i0 += AH) {
+          float mv[AH], sv[AH], xv[AH];
+#pragma unroll
+          for (int k = 0; k < AH; ++k) {
+            const int i = min(i0 + k, n - 2);
+            mv[k] = M[i * n + u];
+            sv[k] = S[i * n + u];
+            xv[k] = Xu[i + 1] * f;
+          }
+#pragma unroll
+          for (int k = 0; k < AH; ++k) {
+            const int i = i0 + k;
+            if (i + 1 < n) {
+              const bool swp = fabsf(sv[k]) < fabsf(e[i]);
+              Xu[i] = swp ? xv[k] : r;
+              r = fmaf(-mv[k], swp ? xv[k] : r, swp ? r : xv[k]);
+            }
+          }
+        }
+      } else {
+        r = eig_noise(n - 1, u);
+      }
+      float x1 = r * ial, x2 = 0.f, nn = x1 * x1;
+      Xu[n - 1] = x1;
+      for (int i0 = n - 2; i0 >= 0; i0 -= AH) {
+        float sv[AH + 1], mp[AH], yv[AH];
+#pragma unroll
+        for (int k = 0; k < AH; ++k) {
+          const int i = max(i0 - k, 0);
+          sv[k] = S[i * n + u];
+          mp[k] = M[max(i - 1, 0) * n + u];
+          yv[k] = it ? Xu[i] : eig_noise(i, u);
+        }
+        sv[AH] = S[max(i0 - AH, 0) * n + u];
+#pragma unroll
+        for (int k = 0; k < AH; ++k) {
+          const int i = i0 - k;
+          if (i >= 0) {
+            const float ei = e[i], en = e[i + 1], ai = sv[k];
+            const bool swp = fabsf(ai) < fabsf(ei), swq = i > 0 && fabsf(sv[k + 1]) < fabsf(e[max(i - 1, 0)]);
+            const float bi = swq ? -mp[k] * ei : ei;
+            const float u0 = swp ? ei : ai, u1 = swp ? d[i + 1] - x : bi, u2 = swp ? en : 0.f;
+            const float xi = fmaf(-u1, x1, fmaf(-u2, x2, yv[k])) * __fdividef(1.f, u0);
+            Xu[i] = xi;
+            nn = fmaf(xi, xi, nn);
+            x2 = x1;
+            x1 = xi;
+          }
+        }
+      }
+      f = rsqrtf(nn);
+    }
+    inorm[u] = f;
+  }
+  tm.sync();
+}
+
+// X <- H_0 ... H_{n-3} X diag(inorm): a 4-lane group holds NV vectors in registers, each
+// lane NC chunks of four consecutive components (16 c + 4 lane ..).
+template <int NC, int NV, bool XS, class Team>
+__device__ __noinline__ void eig_back(const Team tm, const float* A, const float* tau, int n, float* X, int ld,
+                                      const float* inorm) {
+  EIG_SHARED(A);
+  EIG_SHARED(tau);
+  EIG_SHARED(inorm);
+  if (XS) EIG_SHARED(X);
+  const int tr = tm.rank(), ts = tm.size(), lane = threadIdx.x & 31;
+  const int grp = tr >> 2, ngrp = ts >> 2, gl = tr & 3;
+  const unsigned gmask = 0xfu << (lane & 28);
+  for (int u0 = grp; u0 < n; u0 += NV * ngrp) {
+    float4 z[NV][NC];
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+      const int u = u0 + q * ngrp;
+      const float f = u < n ? inorm[u] : 0.f;
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (u < n && 16 * c + 4 * gl < ld) v = *reinterpret_cast<const float4*>(X + u * ld + 16 * c + 4 * gl);
+        z[q][c] = make_float4(v.x * f, v.y * f, v.z * f, v.w * f);
+      }
+    }
+    for (int j = n - 3; j >= 0; --j) {
+      const float t = tau[j];
+      const float* Aj = A + j * ld + 4 * gl;
+      float4 rv[NC];
+      float dt[NV];
+#pragma unroll
+      for (int q = 0; q < NV; ++q) dt[q] = 0.f;
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        rv[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (16 * c + 4 * gl < ld) rv[c] = *reinterpret_cast<const float4*>(Aj + 16 * c);
+      }
+#pragma unroll
+      for (int c = 0; c < NC; ++c)
+#pragma unroll
+        for (int q = 0; q < NV; ++q)
+          dt[q] = fmaf(rv[c].x, z[q][c].x, fmaf(rv[c].y, z[q][c].y, fmaf(rv[c].z, z[q][c].z, fmaf(rv[c].w, z[q][c].w, dt[q]))));
+#pragma unroll
+      for (int o = 2; o > 0; o >>= 1)
+#pragma unroll
+        for (int q = 0; q < NV; ++q) dt[q] += __shfl_xor_sync(gmask, dt[q], o);
+#pragma unroll
+      for (int q = 0; q < NV; ++q) {
+        const float g = -t * dt[q];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          z[q][c].x = fmaf(g, rv[c].x, z[q][c].x);
+          z[q][c].y = fmaf(g, rv[c].y, z[q][c].y);
+          z[q][c].z = fmaf(g, rv[c].z, z[q][c].z);
+          z[q][c].w = fmaf(g, rv[c].w, z[q][c].w);
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+      const int u = u0 + q * ngrp;
+#pragma unroll
+      for (int c = 0; c < NC; ++c)
+        if (u < n && 16 * c + 4 * gl < ld) *reinterpret_cast<float4*>(X + u * ld + 16 * c + 4 * gl) = z[q][c];
+    }
+  }
+  tm.sync();
+}
+
+// Vectors of eigenvalues closer than EIG_CLUSTER (ten times their resolution) to the one before come out of
+// inverse iteration nearly parallel: Gram-Schmidt, twice, within such a run.  Runs are rare
+// and short (the eigenvalues at the rounding level of G); the first warp does it alone.
+constexpr float EIG_CLUSTER = 2e-6f;
+template <bool XS, class Team>
+__device__ __noinline__ void eig_clusters(const Team tm, const float* lam, int n, float* X, int ld) {
+  EIG_SHARED(lam);
+  if (XS) EIG_SHARED(X);
+  const int tr = tm.rank(), lane = threadIdx.x & 31;
+  if (tr < 32) {
+    int start = 0;
+    for (int u = 1; u < n; ++u) {
+      if (lam[u - 1] - lam[u] >= EIG_CLUSTER) {
+        start = u;
+        continue;
+      }
+      float* y = X + u * ld;
+      for (int rep = 0; rep < 2; ++rep) {
+        for (int w = start; w < u; ++w) {
+          const float* x = X + w * ld;
+          float dt = 0.f;
+          for (int i = lane; i < n; i += 32) dt = fmaf(x[i], y[i], dt);
+          dt = warp_sum_f(dt);
+          for (int i = lane; i < n; i += 32) y[i] = fmaf(-dt, x[i], y[i]);
+          __syncwarp();
+        }
+        float nn = 0.f;
+        for (int i = lane; i < n; i += 32) nn = fmaf(y[i], y[i], nn);
+        nn = rsqrtf(fmaxf(warp_sum_f(nn), 1e-20f));
+        for (int i = lane; i < n; i += 32) y[i] *= nn;
+        __syncwarp();
+      }
+    }
+  }
+  tm.sync();
+}
+
+// ----------------------------------------------------------------------------- orthonormalisation
+// E = I - X X^T over the vectors (rows of X; n x n, pad entries zero); returns the largest |entry|.
+template <bool XS, class Team>
+__device__ __noinline__ float eig_defect(const Team tm, const float* X, int n, int ld, float* E) {
+  EIG_SHARED(E);
+  if (XS) EIG_SHARED(X);
+  const int tr = tm.rank(), ts = tm.size();
+  const int nq = (n + 3) >> 2, ntile = nq * (nq + 1) / 2;
+  float worst = 0.f;
+  for (int x = tr; x < n * (ld - n); x += ts) E[(x / (ld - n)) * ld + n + x % (ld - n)] = 0.f;
+  for (int t = tr; t < ntile; t += ts) {
+    int jq = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
+    while (jq * (jq + 1) / 2 > t) --jq;
+    while ((jq + 1) * (jq + 2) / 2 <= t) ++jq;
+    const int iq = t - jq * (jq + 1) / 2;
+    float acc[4][4];
+    const float4* xi[4];
+    const float4* xj[4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      xi[a] = reinterpret_cast<const float4*>(X + min(4 * iq + a, n - 1) * ld);
+      xj[a] = reinterpret_cast<const float4*>(X + min(4 * jq + a, n - 1) * ld);
+#pragma unroll
+      for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
+    }
+    for (int r = 0; r < nq; ++r) {
+      float4 va[4], vb[4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        va[a] = xi[a][r];
+        vb[a] = xj[a][r];
+      }
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+          acc[a][b] = fmaf(va[a].x, vb[b].x, fmaf(va[a].y, vb[b].y, fmaf(va[a].z, vb[b].z, fmaf(va[a].w, vb[b].w, acc[a][b]))));
+    }
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const int i = 4 * iq + a, j = 4 * jq + b;
+        if (i < n && j < n && i <= j) {
+          const float v = (i == j ? 1.f : 0.f) - acc[a][b];
+          worst = (fabsf(v) <= worst) ? worst : fabsf(v);      // NaN stays
+          E[i * ld + j] = v;
+          E[j * ld + i] = v;
+        }
+      }
+  }
+  if (!(worst >= 0.f)) worst = 1e30f;
+  worst = fminf(worst, 1e30f);
+  return tm.max(worst);                            // ends with a team barrier
+}
+// out (row stride lo) = X + E X / 2 over the vectors
+template <bool XS, class Team>
+__device__ __noinline__ void eig_correct(const Team tm, const float* X, const float* E, int n, int ld, float* out, int lo) {
+  EIG_SHARED(E);
+  if (XS) EIG_SHARED(X);
+  const int tr = tm.rank(), ts = tm.size();
+  const int nq = (n + 3) >> 2;
+  for (int t = tr; t < nq * nq; t += ts) {
+    const int iq = t / nq, jq = t % nq;            // vectors 4 iq.., components 4 jq..
+    float acc[4][4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
+#pragma unroll 4
+    for (int k = 0; k < n; ++k) {
+      const float4 x = *reinterpret_cast<const float4*>(X + k * ld + 4 * jq);
+      const float4 y = *reinterpret_cast<const float4*>(E + k * ld + 4 * iq);
+      const float xa[4] = {x.x, x.y, x.z, x.w}, ya[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(ya[a], xa[b], acc[a][b]);
+    }
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const int i = 4 * iq + a, j = 4 * jq + b;
+        if (i < n && j < n) out[i * lo + j] = fmaf(0.5f, acc[a][b], X[i * ld + j]);
+      }
+  }
+  tm.sync();
+}
+
+template <bool XS, class Team>
+__device__ int eig_start_at(const Team tm, const uint4* At, int m, int n, float* A, float* X, float* V, float* Xg,
+                            float* lamg, float* Sg) {
+  const int tr = tm.rank(), ts = tm.size();
+  const int ld = eig_ld(n);
+  float* W = V + 2 * ld;
+  float* P = W + ld;
+  float* d = P + 2 * ld;
+  float* e = d + ld;
+  float* tau = e + ld;
+  float* lam = tau + ld;
+  float* inorm = lam + ld;
+  eig_gram(tm, At, m, n, A, ld);
+  eig_tridiag(tm, A, n, ld, V, W, P, d, e, tau, inorm + ld);
+  const float sc = eig_values(tm, d, e, n, ld, reinterpret_cast<float2*>(P), lam);
+  for (int x = tr; x < n * (ld - n); x += ts) X[(x / (ld - n)) * ld + n + x % (ld - n)] = 0.f;
+  eig_vectors<XS>(tm, d, e, lam, n, X, ld, Sg, Xg, inorm);   // Xg is free until the vectors are finished
+  if (n <= 16) eig_back<1, 2, XS>(tm, A, tau, n, X, ld, inorm);
+  else if (n <= 48) eig_back<3, 2, XS>(tm, A, tau, n, X, ld, inorm);
+  else if (n <= 80) eig_back<5, 2, XS>(tm, A, tau, n, X, ld, inorm);
+  else eig_back<EIG_MAXN / 16, 1, XS>(tm, A, tau, n, X, ld, inorm);
+  eig_clusters<XS>(tm, lam, n, X, ld);
+  const float isc = __fdividef(1.f, sc);
+  for (int u = tr; u < n; u += ts) lamg[u] = fmaxf(lam[u] * isc, 0.f);
+  // Newton-Schulz X <- (3 I - X X^T) X / 2: the defect of inverse iteration is 1e-2 at most for
+  // well separated eigenvalues, up to 1 in clusters
+  for (int it = 0; it < 10; ++it) {
+    const float worst = eig_defect<XS>(tm, X, n, ld, A);
+    if (!(worst < 1.5f)) return 3;
+    eig_correct<XS>(tm, X, A, n, ld, Xg, n);
+    if (worst < 5e-4f) return 0;                   // the defect after the correction is its square
+    for (int x = tr; x < n * n; x += ts) X[(x / n) * ld + x % n] = Xg[x];
+    tm.sync();
+  }
+  return 3;
+}
+// Approximate eigenvectors and eigenvalues of B^T B.  At: the digits of B^T (eig_digits); arena:
+// `words` floats of shared memory (16-byte aligned); Xg (n x n floats, row stride n, one
+// vector per row, eigenvalues descending) and lamg (n floats) receive the result, Sg (n x
+// n floats) and Xalt (n x ld floats, for X where the arena only holds A) are scratch, all
+// in global memory.  Returns 0, 1 if the block does not fit (no result), or 3 if X is not
+// orthonormal in the end (the eigenvalues hold).
+template <class Team>
+__device__ int eig_start(const Team& tm, const uint4* At, int m, int n, float* arena, int words, float* Xg, float* lamg,
+                         float* Sg, float* Xalt) {
+  const int ld = eig_ld(n);
+  if (n > EIG_MAXN || n * ld + eig_vec_floats(n) > words) return 1;
+  if (2 * n * ld + eig_vec_floats(n) <= words)
+    return eig_start_at<true>(tm, At, m, n, arena, arena + n * ld, arena + 2 * n * ld, Xg, lamg, Sg);
+  return eig_start_at<false>(tm, At, m, n, arena, Xalt, arena + n * ld, Xg, lamg, Sg);
+}
+
+// ----------------------------------------------------------------------------- refinement
+// W (column k at k ldw, rows padded to 16) = B X from the digits of B (A) and of X (D): NA, NB, NS
+// as for mma_tile.
+template <int NA, int NB, int NS, class Team>
+__device__ __noinline__ void eig_bx(const Team tm, const uint4* A, const uint2* D, int m, int n, int kp, float2* W,
+                                    int ldw) {
+  const int lane = threadIdx.x & 31, warp = tm.rank() >> 5, nw = tm.size() >> 5;
+  const int mt = pad16(m) >> 4, KT = pad16(n) >> 4, JT = kp >> 3, g = lane >> 2, t2 = 2 * (lane & 3);
+  for (int t = warp; t < mt * JT; t += nw) {
+    const int it = t % mt, j = t / mt;
+    float acc[NS - 1][4];
+    mma_tile<NA, NB, NS>(A, D, it, j, KT, JT, lane, acc);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      W[(size_t)(8 * j + t2 + (q & 1)) * ldw + 16 * it + g + 8 * (q >> 1)] = mma_value<NS>(acc, q, 0);
+  }
+  tm.sync();
+}
+// R (column k at k ld) = B^T W - X lambda from the digits of B^T (At) and of W (D).
+template <int NA, int NB, int NS, class Team>
+__device__ __noinline__ void eig_residual(const Team tm, const uint4* At, const uint2* D, int m, int n, int kp,
+                                          const float2* Xd, int ldx, const float2* lk, float* R, int ld) {
+  EIG_SHARED(lk);
+  EIG_SHARED(R);
+  const int lane = threadIdx.x & 31, warp = tm.rank() >> 5, nw = tm.size() >> 5;
+  const int nt = pad16(n) >> 4, KT = pad16(m) >> 4, JT = kp >> 3, g = lane >> 2, t2 = 2 * (lane & 3);
+  for (int t = warp; t < nt * JT; t += nw) {
+    const int it = t % nt, j = t / nt;
+    float2 xv[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) xv[q] = Xd[(size_t)(8 * j + t2 + (q & 1)) * ldx + 16 * it + g + 8 * (q >> 1)];
+    float acc[NS - 1][4];
+    mma_tile<NA, NB, NS>(At, D, it, j, KT, JT, lane, acc);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int k = 8 * j + t2 + (q & 1), c = 16 * it + g + 8 * (q >> 1);
+      const float2 lx = dfa::mul(lk[k], xv[q]);
+      const float2 df = dfa::add(mma_value<NS>(acc, q, EIG_WEXP), make_float2(-lx.x, -lx.y));
+      if (c < ld) R[k * ld + c] = c < n ? df.x + df.y : 0.f;
+    }
+  }
+  tm.sync();
+}
+// |column k|^2 of V (column k at k ldv, length K) as a double-float: eight lanes per column; f(k, value)
+// runs on one lane.
+template <class Team, class F>
+__device__ __forceinline__ void eig_norms(const Team& tm, const float2* V, int ldv, int K, int kp, F f) {
+  const int lane = threadIdx.x & 31, warp = tm.rank() >> 5, nw = tm.size() >> 5;
+  for (int t = warp; t < kp / 4; t += nw) {
+    const int k = 4 * t + (lane >> 3);
+    const float2* src = V + (size_t)k * ldv;
+    float s = 0.f, er = 0.f;
+#pragma unroll 4
+    for (int r = lane & 7; r < K; r += 8) {
+      const float2 v = src[r];
+      dot2_step(v, v, s, er);
+    }
+    float2 l = df_pair(s, er);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1)
+      l = dfa::add(l, make_float2(__shfl_xor_sync(0xffffffffu, l.x, o), __shfl_xor_sync(0xffffffffu, l.y, o)));
+    if ((lane & 7) == 0) f(k, l);
+  }
+}
+// T (row i at i kp) = X R / (lambda_k - lambda_i), half the norm's defect ek on the diagonal: lanes are
+// vectors i.  Returns the largest |entry|.
+template <class Team>
+__device__ __noinline__ float eig_angles(const Team tm, const float* X, const float* R, int n, int ld, int kc, int kp,
+                                         const float2* lk, const float* ek, const float* lam, float* T) {
+  EIG_SHARED(R);
+  EIG_SHARED(lk);
+  EIG_SHARED(ek);
+  EIG_SHARED(lam);
+  EIG_SHARED(T);
+  const int lane = threadIdx.x & 31, warp = tm.rank() >> 5, nw = tm.size() >> 5;
+  const int rc = (n + 31) >> 5, kcn = kp / EIG_TC, nq = (n + 3) >> 2;
+  float worst = 0.f;
+  for (int t = warp; t < rc * kcn; t += nw) {
+    const int i = (t % rc) * 32 + lane, k0 = (t / rc) * EIG_TC;
+    float s[EIG_TC];
+#pragma unroll
+    for (int q = 0; q < EIG_TC; ++q) s[q] = 0.f;
+    const float4* xp = reinterpret_cast<const float4*>(X + min(i, n - 1) * ld);
+    const float4* rp = reinterpret_cast<const float4*>(R + k0 * ld);
+    const int l4 = ld >> 2;
+#pragma unroll 2
+    for (int c = 0; c < nq; ++c) {
+      const float4 x = xp[c];
+#pragma unroll
+      for (int q = 0; q < EIG_TC; ++q) {
+        const float4 r = rp[q * l4 + c];
+        s[q] = fmaf(x.x, r.x, fmaf(x.y, r.y, fmaf(x.z, r.z, fmaf(x.w, r.w, s[q]))));
+      }
+    }
+    if (i < n) {
+      const float2 li = i < kc ? lk[i] : make_float2(lam[i], 0.f);
+      float o[EIG_TC];
+#pragma unroll
+      for (int q = 0; q < EIG_TC; ++q) {
+        const int k = k0 + q;
+        float v = 0.f;
+        if (k < kc) {
+          if (i == k) {
+            v = 0.5f * ek[k];
+          } else {
+            const float den = (lk[k].x - li.x) + (lk[k].y - li.y);
+            v = den != 0.f ? __fdividef(s[q], den) : (s[q] == 0.f ? 0.f : 1e30f);
+          }
+          worst = (fabsf(v) <= worst) ? worst : fabsf(v);
+        }
+        o[q] = v;
+      }
+      *reinterpret_cast<float4*>(T + i * kp + k0) = make_float4(o[0], o[1], o[2], o[3]);
+      *reinterpret_cast<float4*>(T + i * kp + k0 + 4) = make_float4(o[4], o[5], o[6], o[7]);
+    }
+  }
+  if (!(worst >= 0.f)) worst = 1e30f;
+  return tm.max(fminf(worst, 1e30f));
+}
+// Xd (column k at k ldx) += X^T T, and the FP32 vectors Xg (row k at k n) follow: lanes are components.
+template <class Team>
+__device__ __noinline__ void eig_update(const Team tm, const float* X, const float* T, int n, int ld, int kc, int kp,
+                                        float2* Xd, int ldx, float* Xg) {
+  EIG_SHARED(T);
+  const int lane = threadIdx.x & 31, warp = tm.rank() >> 5, nw = tm.size() >> 5;
+  const int rc = (n + 31) >> 5, kcn = kp / EIG_TC;
+  for (int t = warp; t < rc * kcn; t += nw) {
+    const int i = (t % rc) * 32 + lane, k0 = (t / rc) * EIG_TC, ic = min(i, n - 1);
+    float s[EIG_TC];
+    float2 xv[EIG_TC];
+#pragma unroll
+    for (int q = 0; q < EIG_TC; ++q) {
+      s[q] = 0.f;
+      xv[q] = Xd[(size_t)(k0 + q) * ldx + ic];
+    }
+    const float* xp = X + ic;
+#pragma unroll 4
+    for (int v = 0; v < n; ++v) {
+      const float x = xp[v * ld];
+      const float4 ra = *reinterpret_cast<const float4*>(T + v * kp + k0);
+      const float4 rb = *reinterpret_cast<const float4*>(T + v * kp + k0 + 4);
+      s[0] = fmaf(x, ra.x, s[0]);
+      s[1] = fmaf(x, ra.y, s[1]);
+      s[2] = fmaf(x, ra.z, s[2]);
+      s[3] = fmaf(x, ra.w, s[3]);
+      s[4] = fmaf(x, rb.x, s[4]);
+      s[5] = fmaf(x, rb.y, s[5]);
+      s[6] = fmaf(x, rb.z, s[6]);
+      s[7] = fmaf(x, rb.w, s[7]);
+    }
+    if (i < n) {
+#pragma unroll
+      for (int q = 0; q < EIG_TC; ++q) {
+        const float2 v = dfa::add(xv[q], make_float2(s[q], 0.f));
+        Xd[(size_t)(k0 + q) * ldx + i] = v;
+        if (k0 + q < kc) Xg[(k0 + q) * n + i] = v.x;
+      }
+    }
+  }
+  tm.sync();
+}
+
+// Refines the first kc vectors of Xg (n x n, one per row; updated) as described at the top.  A, At: the
+// digits of B and B^T; lam0 the approximate eigenvalues.  Outputs: Wout (column j at j m), Qout
+// (column j at j n) in FP64, the singular values in sig[0..kc).  Wd, Xd (kp columns of length m
+// and n padded to 16, double-floats), Dg (digits of either) and Xalt (n x ld floats) are global
+// scratch; the last two are used where the arena is too small.  Returns 0, or 1 if the
+// corrections do not converge or the block does not fit.
+template <class Team>
+__device__ int eig_refine(const Team& tm, const uint4* A, const uint4* At, int m, int n, int kc, float* Xg,
+                          const float* lam0, float* arena, int words, float2* Wd, float2* Xd, uint2* Dg, float* Xalt,
+                          double* Wout, double* Qout, double* sig, double scale) {
+  const int tr = tm.rank(), ts = tm.size();
+  const int ld = eig_ld(n), kp = eig_kp(kc), m16 = pad16(m), n16 = pad16(n);
+  // arena: lk (kp float2), ek (kp), lam (ld), R (kp x ld), then the digits or, after them, T (n x kp) and X (n x ld)
+  const int fix = 3 * kp + ld + kp * ld, dig = m16 * kp * EIG_DIG / 2, tx = n * kp;
+  if (fix + tx > words) return 1;
+  float2* lk = reinterpret_cast<float2*>(arena);
+  float* ek = arena + 2 * kp;
+  float* lam = ek + kp;
+  float* R = lam + ld;
+  float* T = R + kp * ld;
+  uint2* D = fix + dig <= words ? reinterpret_cast<uint2*>(T) : Dg;
+  const bool xin = fix + tx + n * ld <= words;
+  float* X = xin ? T + tx : Xalt;
+  for (int x = tr; x < n16 * kp; x += ts) {
+    const int k = x / n16, c = x % n16;
+    float v = (k < kc && c < n) ? Xg[k * n + c] : 0.f;
+    // four digits carry the start vectors: entries below 2^-7 are rounded to 2^-30
+    if (fabsf(v) < 0.0078125f) v = __fsub_rn(__fadd_rn(v, 0.01171875f), 0.01171875f);
+    Xd[x] = make_float2(v, 0.f);
+  }
+  for (int x = tr; x < n; x += ts) lam[x] = lam0[x];
+  tm.sync();
+  for (int it = 0; it < 6; ++it) {
+    // the first correction starts from 1e-6 and needs 1e-10: six digits of B, four of X
+    if (it == 0) {
+      eig_digits_cols<4>(tm, Xd, n16, n, kp, 0, D);
+      eig_bx<6, 4, 7>(tm, A, D, m, n, kp, Wd, m16);
+    } else {
+      eig_digits_cols<EIG_DIG>(tm, Xd, n16, n, kp, 0, D);
+      eig_bx<EIG_DIG, EIG_DIG, EIG_DIG + 1>(tm, A, D, m, n, kp, Wd, m16);
+    }
+    eig_norms(tm, Wd, m16, m, kp, [&](int k, float2 l) {
+      lk[k] = l;
+      if (k < kc) lam[k] = l.x;
+    });
+    eig_norms(tm, Xd, n16, n, kp, [&](int k, float2 l) { ek[k] = __fadd_rn(__fadd_rn(1.f, -l.x), -l.y); });
+    tm.sync();
+    if (it == 0) {
+      eig_digits_cols<6>(tm, Wd, m16, m, kp, EIG_WEXP, D);
+      eig_residual<6, 6, 7>(tm, At, D, m, n, kp, Xd, n16, lk, R, ld);
+    } else {
+      eig_digits_cols<EIG_DIG>(tm, Wd, m16, m, kp, EIG_WEXP, D);
+      eig_residual<EIG_DIG, EIG_DIG, EIG_DIG + 1>(tm, At, D, m, n, kp, Xd, n16, lk, R, ld);
+    }
+    for (int x = tr; x < n * ld; x += ts) {
+      const int u = x / ld, c = x % ld;
+      X[x] = c < n ? Xg[u * n + c] : 0.f;
+    }
+    tm.sync();
+    const float worst = eig_angles(tm, X, R, n, ld, kc, kp, lk, ek, lam, T);
+    if (!(worst < 0.05f)) return 1;
+    eig_update(tm, X, T, n, ld, kc, kp, Xd, n16, Xg);
+    if (worst <= 1e-8f) break;
+    if (it == 5) return 1;
+  }
+  eig_digits_cols<EIG_DIG>(tm, Xd, n16, n, kp, 0, D);
+  eig_bx<EIG_DIG, EIG_DIG, EIG_DIG + 1>(tm, A, D, m, n, kp, Wd, m16);
+  eig_norms(tm, Wd, m16, m, kp, [&](int k, float2 l) {
+    if (k < kc) sig[k] = sqrt(dfa::to_double(l)) * scale;
+  });
+  for (int x = tr; x < m * kc; x += ts) Wout[x] = dfa::to_double(Wd[(size_t)(x / m) * m16 + x % m]);
+  for (int x = tr; x < n * kc; x += ts) Qout[x] = dfa::to_double(Xd[(size_t)(x / n) * n16 + x % n]);
+  tm.sync();
+  return 0;
+}
+
+}  // namespace
+}  // namespace tnqe
