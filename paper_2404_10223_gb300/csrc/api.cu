@@ -561,6 +561,8 @@ void run_rotations(tnqe_ctx* c, const std::vector<std::pair<int, int>>& pairs, R
     d.q32 = d.w32 + blk;
     d.frag = reinterpret_cast<uint4*>(d.tbuf + 2 * blk);
     d.xchg = d.tbuf + 2 * blk + rb.tiles[k] * ROT_TILE_DOUBLES;
+    d.carve = nullptr;
+    d.carve_cap = 0;
     d.meta = c->rot_meta.as<int>() + META_INTS * cluster * k;
     d.meta_cap = META_INTS;
     d.discarded = ddisc;

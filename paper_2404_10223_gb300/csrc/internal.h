@@ -90,6 +90,8 @@ struct RotDesc {
   float* w32;                     // FP32 working copy of each block
   float* q32;                     // FP32 singular vectors of each block
   void* xchg;                     // exchange area of the pair's CTAs (ROT_XCHG_BYTES)
+  double* carve;                  // not NULL: lay the block buffers out here per gate, carve_cap doubles
+  long long carve_cap;
   int* meta;                      // scratch ints, meta_cap for each CTA of the pair
   long long meta_cap;
   double* discarded;

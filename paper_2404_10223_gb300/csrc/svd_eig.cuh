@@ -74,6 +74,18 @@ __host__ __device__ __forceinline__ int eig_vec_floats(int n) { return 11 * eig_
 // Tells the compiler that a generic pointer points to shared memory.
 #define EIG_SHARED(p) __builtin_assume(__isShared(p))
 
+// Two FP32 multiply-adds in one instruction.
+__device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
+  unsigned long long x, y, z, r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a.x), "f"(a.y));
+  asm("mov.b64 %0, {%1, %2};" : "=l"(y) : "f"(b.x), "f"(b.y));
+  asm("mov.b64 %0, {%1, %2};" : "=l"(z) : "f"(c.x), "f"(c.y));
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(x), "l"(y), "l"(z));
+  float2 o;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(o.x), "=f"(o.y) : "l"(r));
+  return o;
+}
+
 // s + e accumulates a b (double-floats): the compensated dot product of Ogita, Rump
 // and Oishi (SIAM J. Sci. Comput. 26 (2005) 1955), as accurate as twice FP32.
 __device__ __forceinline__ void dot2_step(float2 a, float2 b, float& s, float& e) {
@@ -165,17 +177,18 @@ __device__ __noinline__ void eig_digits(const Team tm, const double* raw, int m,
   const int mt = pad16(m) >> 4, nt = pad16(n) >> 4, g = lane >> 2, t2 = 2 * (lane & 3);
   for (int t = warp; t < mt * nt; t += nw) {
     const int it = t % mt, kt = t / mt;
-    long long v[4][2];                             // registers (rows g, g + 8) x (columns t2, t2 + 8), pairs along the row
+    double v[4][2];                                // registers (rows g, g + 8) x (columns t2, t2 + 8), pairs along the row
 #pragma unroll
     for (int q = 0; q < 4; ++q)
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int r = 16 * it + g + 8 * (q & 1), c = 16 * kt + t2 + 8 * (q >> 1) + h;
-        v[q][h] = (r < m && c < n) ? fix_double(raw[(size_t)c * m + r], ex) : 0;
+        const double x = raw[(size_t)min(c, n - 1) * m + min(r, m - 1)];
+        v[q][h] = (r < m && c < n) ? x : 0.0;
       }
     unsigned w[4][EIG_DIG];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) digits_pair(v[q][0], v[q][1], w[q]);
+    for (int q = 0; q < 4; ++q) digits_pair(fix_double(v[q][0], ex), fix_double(v[q][1], ex), w[q]);
     uint4* a = A + (size_t)(it * nt + kt) * EIG_DIG * 32 + lane;
     uint4* b = At + (size_t)(kt * mt + it) * EIG_DIG * 32 + lane;
 #pragma unroll
@@ -210,7 +223,9 @@ __device__ __noinline__ void eig_digits_cols(const Team tm, const float2* V, int
 
 // One 16 x 8 tile of the product: NA digits of the first operand (tile row `it`, KT tiles), NB of the
 // second (tile column j of JT), products of order up to NS.  acc[o] holds the sums of order
-// o + 2 in units of 2^(4 - 8 (o + 2)).
+// o + 2 in units of 2^(4 - 8 (o + 2)).  The first operand comes from L2, one tile ahead of
+// its use.  (Two tiles sharing its loads, without that: 96.0 against 91.6 ms of rotation on
+// N = 14, chi = 128.)
 template <int NA, int NB, int NS>
 __device__ __forceinline__ void mma_tile(const uint4* A, const uint2* D, int it, int j, int KT, int JT, int lane,
                                          float (&acc)[NS - 1][4]) {
@@ -306,44 +321,40 @@ __device__ __noinline__ void eig_gram(const Team tm, const uint4* At, int m, int
 
 // ----------------------------------------------------------------------------- tridiagonalisation
 // Householder reduction of the symmetric A (row stride ld): diagonal d, off-diagonal
-// e, reflectors I - tau v v^T with v left in row j of A (zero up to column j).
+// e, reflectors I - tau v v^T; reflector t is left in row t - 1 of A, the first in V
+// (zero up to component t).
 //
-// Latency bound: n - 2 dependent steps, so a step has one team barrier and one
-// reduction.  The rows of the trailing matrix belong to 8-lane groups; a group applies
-// the last rank-2 update to its rows and multiplies them with the new reflector in one
-// pass.  Every warp forms the reflector of row t by itself, from the row in memory,
-// the products p = tau A v of the last step and the last reflector v (v_t = 1):
+// n - 2 dependent steps with one team barrier and one reduction each; bound by the
+// instructions of a step where four teams share an SM, by their latency otherwise.  The
+// rows of the trailing matrix belong to 8-lane groups; a group applies the last rank-2
+// update to its rows and multiplies them with the new reflector in one pass, two rows
+// at a time, in packed FP32 pairs.  Every warp forms the reflector of row t by itself,
+// from the row in memory, the products p = tau A v of the last step and the last
+// reflector v (v_t = 1):
 //   w = p - K v, K = tau p.v / 2,   row t of A - v w^T - w v^T  =  u + kappa v,
 //   u = a - p, kappa = 2 K - p_t,
 // so that K and the norm of the row come from sums over p, u and v that do not wait
-// for one another (where they cancel, the norm is summed again).  V (two, by parity),
-// W and P (two) hold v, w, p; all warps write the same values into V and W.
+// for one another (where they cancel, the norm is summed again).  W and P (two, by
+// parity) hold w and p; all warps write the same values into the reflectors and W.
 template <int NE, class Team>
 __device__ __noinline__ void eig_tridiag_ne(const Team tm, float* A, int n, int ld, float* V, float* W, float* P, float* d,
                                             float* e, float* tau, float* dummy) {
   // 32-bit offsets into the pool: a pointer select per row would cost 64-bit arithmetic
   extern __shared__ float4 rot_pool[];
   float* const S = reinterpret_cast<float*>(rot_pool);
-  const int Vo = (int)(V - S), Wo = (int)(W - S), Ao = (int)(A - S), Do = (int)(dummy - S);
-  A = S + Ao;
-  V = S + Vo;
-  W = S + Wo;
-  P = S + (int)(P - S);
-  d = S + (int)(d - S);
-  e = S + (int)(e - S);
-  tau = S + (int)(tau - S);
-  dummy = S + Do;
+  const int Vo = (int)(V - S), Wo = (int)(W - S), Ao = (int)(A - S), Po = (int)(P - S), Do = (int)(dummy - S);
+  const int so = (int)(d - S), eo = (int)(e - S), to = (int)(tau - S);
   const int tr = tm.rank(), ts = tm.size();
   const int lane = threadIdx.x & 31, grp = tr >> 3, ngrp = ts >> 3, gl = tr & 7;
   const unsigned gmask = 0xffu << ((lane >> 3) * 8);
-  const bool first = tr < 32;
+  const bool one = tr == 0;
   for (int c = tr; c < ld; c += ts) {
-    V[c] = 0.f;
-    V[ld + c] = 0.f;
-    W[c] = 0.f;
-    P[c] = 0.f;
-    P[ld + c] = 0.f;
-    dummy[c] = 0.f;                                // stays finite: its products meet zeros
+    S[Vo + c] = 0.f;
+    S[Vo + ld + c] = 0.f;                          // the reflector before the first
+    S[Wo + c] = 0.f;
+    S[Po + c] = 0.f;
+    S[Po + ld + c] = 0.f;
+    S[Do + c] = 0.f;                               // stays finite: its products meet zeros
   }
   tm.sync();
   float v[NE];
@@ -351,28 +362,24 @@ __device__ __noinline__ void eig_tridiag_ne(const Team tm, float* A, int n, int 
   int rfirst = grp;                                // the group's first row of the trailing matrix
 #pragma unroll
   for (int q = 0; q < NE; ++q) v[q] = 0.f;
+  int vp = Vo + ld, vc = Vo;                       // the last and the new reflector
+#pragma unroll 1
   for (int t = 0; t + 1 < n; ++t) {
-    float* Vc = V + (t & 1) * ld;                  // this step's reflector
-    const float* Vp = V + ((t & 1) ^ 1) * ld;      // the last one
-    float* Pc = P + (t & 1) * ld;
-    const float* Pp = P + ((t & 1) ^ 1) * ld;
-    const float* Ar = A + t * ld;
-    const float pt = Pp[t], at = Ar[t];
-    const float an = Ar[t + 1], pn = Pp[t + 1], vnx = Vp[t + 1];
+    const int pc = Po + (t & 1) * ld, pp = Po + ((t & 1) ^ 1) * ld, ar = Ao + t * ld;
+    const float pt = S[pp + t], at = S[ar + t];
+    const float an = S[ar + t + 1], pn = S[pp + t + 1], vn = S[vp + t + 1];
     float p[NE], u[NE];
     float s1 = 0.f, s2 = 0.f, s3 = 0.f, s4 = 0.f;
 #pragma unroll
     for (int q = 0; q < NE; ++q) {
-      const int c = lane + 32 * q;
-      const bool in = c >= t && c < n;
-      p[q] = in ? Pp[c] : 0.f;
-      u[q] = in ? Ar[c] - p[q] : 0.f;
+      const int c = lane + 32 * q, cc = NE == 1 || c < ld ? c : 0;
+      p[q] = c < ld ? S[pp + cc] : 0.f;            // v is zero before t and from n on
+      u[q] = c < ld ? S[ar + cc] - p[q] : 0.f;
       s1 = fmaf(p[q], v[q], s1);
-      if (c > t + 1) {
-        s2 = fmaf(u[q], u[q], s2);
-        s3 = fmaf(u[q], v[q], s3);
-        s4 = fmaf(v[q], v[q], s4);
-      }
+      const float um = c > t + 1 ? u[q] : 0.f, vm = c > t + 1 ? v[q] : 0.f;
+      s2 = fmaf(um, um, s2);
+      s3 = fmaf(um, vm, s3);
+      s4 = fmaf(vm, vm, s4);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -382,27 +389,26 @@ __device__ __noinline__ void eig_tridiag_ne(const Team tm, float* A, int n, int 
       s4 += __shfl_xor_sync(0xffffffffu, s4, o);
     }
     const float K = 0.5f * tl * s1, kap = 2.f * K - pt;
-    const float x0 = fmaf(kap, vnx, an - pn);
+    const float x0 = fmaf(kap, vn, an - pn);
     if (t + 2 == n) {                              // the last 2 x 2 block needs no reflector
-      if (first && lane == 0) {
+      if (one) {
         const int c = n - 1;
-        const float vl = Vp[c], wl = fmaf(-K, vl, Pp[c]);
-        d[t] = at - pt + kap;
-        e[t] = x0;
-        d[c] = A[c * ld + c] - 2.f * vl * wl;
+        const float vl = S[vp + c], wl = fmaf(-K, vl, S[pp + c]);
+        S[so + t] = at - pt + kap;
+        S[eo + t] = x0;
+        S[so + c] = S[Ao + c * ld + c] - 2.f * vl * wl;
       }
       break;
     }
-    float x[NE];
-#pragma unroll
-    for (int q = 0; q < NE; ++q) x[q] = fmaf(kap, v[q], u[q]);
     const float big = fmaf(kap * kap, s4, s2);
     s2 = fmaf(kap, fmaf(kap, s4, 2.f * s3), s2);
     if (s2 < 0.02f * big) {                        // the sums cancelled
       s2 = 0.f;
 #pragma unroll
-      for (int q = 0; q < NE; ++q)
-        if (lane + 32 * q > t + 1) s2 = fmaf(x[q], x[q], s2);
+      for (int q = 0; q < NE; ++q) {
+        const float x = fmaf(kap, v[q], u[q]);
+        if (lane + 32 * q > t + 1) s2 = fmaf(x, x, s2);
+      }
       s2 = warp_sum_f(s2);
     }
     float tj = 0.f, beta = x0, inv = 0.f;
@@ -415,86 +421,73 @@ __device__ __noinline__ void eig_tridiag_ne(const Team tm, float* A, int n, int 
 #pragma unroll
     for (int q = 0; q < NE; ++q) {
       const int c = lane + 32 * q;
-      const float w = fmaf(-K, v[q], p[q]);
-      v[q] = (c == t + 1) ? 1.f : ((c > t + 1) ? x[q] * inv : 0.f);
+      const float w = fmaf(-K, v[q], p[q]), x = fmaf(kap, v[q], u[q]) * inv;
+      v[q] = (c == t + 1) ? 1.f : ((c > t + 1) ? x : 0.f);
       if (c < ld) {
-        W[c] = w;
-        Vc[c] = v[q];
+        S[Wo + c] = w;
+        S[vc + c] = v[q];
       }
+    }
+    if (one) {
+      S[so + t] = at - pt + kap;
+      S[eo + t] = beta;
+      S[to + t] = tj;
     }
     __syncwarp();
-    // rows t + 1.. of the trailing matrix: the last update, and the product with the
-    // reflector, four rows at a time without branches (what lies outside goes to a dummy row)
-    const int c0 = (t + 1) & ~3;
+    // rows t + 1.. of the trailing matrix: the last update, and the product with the new
+    // reflector (what lies outside goes to a dummy row)
+    const int c0 = ((t + 1) & ~3) + 4 * gl;
     if (rfirst < t + 1) rfirst += ngrp;
-    for (int r = rfirst; r < n; r += 4 * ngrp) {
-      float acc[4], vr[4], wr[4];
-      int R[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int ri = r + i * ngrp, rc = min(ri, n - 1);
-        vr[i] = Vp[rc];
-        wr[i] = W[rc];
-        R[i] = ri < n ? Ao + ri * ld : Do;
-        acc[i] = 0.f;
+#pragma unroll 1
+    for (int r = rfirst; r < n; r += 2 * ngrp) {
+      const int r2 = r + ngrp, rb = r2 < n ? r2 : r;
+      const float va = -S[vp + r], wa = -S[Wo + r], vb = -S[vp + rb], wb = -S[Wo + rb];
+      const int Ra = Ao + r * ld, Rb = r2 < n ? Ao + r2 * ld : Do;
+      const float2 va2 = make_float2(va, va), wa2 = make_float2(wa, wa), vb2 = make_float2(vb, vb), wb2 = make_float2(wb, wb);
+      float2 sa = make_float2(0.f, 0.f), sb = sa;
+#pragma unroll 1
+      for (int c = c0; c < ld; c += 32) {
+        const float4 vq = *reinterpret_cast<const float4*>(S + vp + c), wq = *reinterpret_cast<const float4*>(S + Wo + c);
+        const float4 nq = *reinterpret_cast<const float4*>(S + vc + c);
+        float4 xa = *reinterpret_cast<const float4*>(S + Ra + c), xb = *reinterpret_cast<const float4*>(S + Rb + c);
+        const float2 v0 = make_float2(vq.x, vq.y), v1 = make_float2(vq.z, vq.w), w0 = make_float2(wq.x, wq.y),
+                     w1 = make_float2(wq.z, wq.w), n0 = make_float2(nq.x, nq.y), n1 = make_float2(nq.z, nq.w);
+        const float2 a0 = ffma2(va2, w0, ffma2(wa2, v0, make_float2(xa.x, xa.y)));
+        const float2 a1 = ffma2(va2, w1, ffma2(wa2, v1, make_float2(xa.z, xa.w)));
+        const float2 b0 = ffma2(vb2, w0, ffma2(wb2, v0, make_float2(xb.x, xb.y)));
+        const float2 b1 = ffma2(vb2, w1, ffma2(wb2, v1, make_float2(xb.z, xb.w)));
+        *reinterpret_cast<float4*>(S + Ra + c) = make_float4(a0.x, a0.y, a1.x, a1.y);
+        *reinterpret_cast<float4*>(S + Rb + c) = make_float4(b0.x, b0.y, b1.x, b1.y);
+        sa = ffma2(a0, n0, ffma2(a1, n1, sa));
+        sb = ffma2(b0, n0, ffma2(b1, n1, sb));
       }
-      for (int cb = c0; cb < ld; cb += 32) {
-        const bool in = cb + 4 * gl < ld;
-        const int c = in ? cb + 4 * gl : 0;
-        const float4 vp = *reinterpret_cast<const float4*>(Vp + c), wp = *reinterpret_cast<const float4*>(W + c);
-        float4 vc = *reinterpret_cast<const float4*>(Vc + c);
-        float4 a[4];
-        int to[4];
+      float ya = sa.x + sa.y, yb = sb.x + sb.y;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          to[i] = in ? R[i] + c : Do;
-          a[i] = *reinterpret_cast<const float4*>(S + to[i]);
-        }
-        if (!in) vc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          a[i].x = fmaf(-vr[i], wp.x, fmaf(-wr[i], vp.x, a[i].x));
-          a[i].y = fmaf(-vr[i], wp.y, fmaf(-wr[i], vp.y, a[i].y));
-          a[i].z = fmaf(-vr[i], wp.z, fmaf(-wr[i], vp.z, a[i].z));
-          a[i].w = fmaf(-vr[i], wp.w, fmaf(-wr[i], vp.w, a[i].w));
-          *reinterpret_cast<float4*>(S + to[i]) = a[i];
-          acc[i] = fmaf(a[i].x, vc.x, fmaf(a[i].y, vc.y, fmaf(a[i].z, vc.z, fmaf(a[i].w, vc.w, acc[i]))));
-        }
+      for (int o = 4; o > 0; o >>= 1) {
+        ya += __shfl_xor_sync(gmask, ya, o);
+        yb += __shfl_xor_sync(gmask, yb, o);
       }
-#pragma unroll
-      for (int o = 4; o > 0; o >>= 1)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) acc[i] += __shfl_xor_sync(gmask, acc[i], o);
-      // lane i of the group stores the product of row i
-      const float mine = gl == 0 ? acc[0] : (gl == 1 ? acc[1] : (gl == 2 ? acc[2] : acc[3]));
-      if (gl < 4 && r + gl * ngrp < n) Pc[r + gl * ngrp] = tj * mine;
+      if (gl == 0) S[pc + r] = tj * ya;
+      if (gl == 1 && r2 < n) S[pc + r2] = tj * yb;
     }
     tm.sync();
-    if (first) {                                   // no other warp reads row t any more
-#pragma unroll
-      for (int q = 0; q < NE; ++q)
-        if (lane + 32 * q < ld) A[t * ld + lane + 32 * q] = v[q];
-      if (lane == 0) {
-        d[t] = at - pt + kap;
-        e[t] = beta;
-        tau[t] = tj;
-      }
-    }
     tl = tj;
+    vp = vc;
+    vc = Ao + t * ld;                              // row t is dead now
   }
-  if (n == 1 && tr == 0) d[0] = A[0];
+  if (n == 1 && one) S[so] = S[Ao];
   tm.sync();
 }
-// More than four warps (eight from n = 97 on) only add redundant work to the steps.
+// More than four warps (two up to n = 48, eight from n = 97 on) only add redundant work to the steps.
 template <class Team>
 __device__ void eig_tridiag(const Team& tm, float* A, int n, int ld, float* V, float* W, float* P, float* d, float* e,
                             float* tau, float* dummy) {
-  const auto sub = tm.part(n <= 96 ? 128 : 256);
+  const auto sub = tm.part(n <= 48 ? 64 : (n <= 96 ? 128 : 256));
   if (sub.rank() < sub.size()) {
-    if (n <= 32) eig_tridiag_ne<1>(sub, A, n, ld, V, W, P, d, e, tau, dummy);
-    else if (n <= 64) eig_tridiag_ne<2>(sub, A, n, ld, V, W, P, d, e, tau, dummy);
-    else if (n <= 96) eig_tridiag_ne<3>(sub, A, n, ld, V, W, P, d, e, tau, dummy);
-    else eig_tridiag_ne<EIG_NE>(sub, A, n, ld, V, W, P, d, e, tau, dummy);
+    if (n <= 28) eig_tridiag_ne<1>(sub, A, n, ld, V, W, P, d, e, tau, dummy);
+    else if (n <= 60) eig_tridiag_ne<2>(sub, A, n, ld, V, W, P, d, e, tau, dummy);
+    else if (n <= 92) eig_tridiag_ne<3>(sub, A, n, ld, V, W, P, d, e, tau, dummy);
+    else eig_tridiag_ne<EIG_NE + 1>(sub, A, n, ld, V, W, P, d, e, tau, dummy);
   }
   tm.sync();
 }
@@ -582,12 +575,12 @@ __device__ __noinline__ float eig_values(const Team tm, float* d, float* e, int 
 // One thread per vector: LU with partial pivoting of T - lam, then two steps of inverse
 // iteration; the first starts from a generic right-hand side after the forward
 // elimination, so it is a back substitution alone.  X[u * ld + i] is component i of
-// vector u; S and M (n x n, row stride n, global memory) keep the pivots and the
-// multipliers, read eight rows ahead of their use.  A row swap at step i shows as
-// |pivot_i| < |e_i|.  inorm[u] gets 1 / |vector u|.
+// vector u; SM (n x n pairs, row stride n, global memory) keeps the pivots and the
+// multipliers, loaded eight rows ahead of the eight in use (L2 latency).  A row swap at
+// step i shows as |pivot_i| < |e_i|.  inorm[u] gets 1 / |vector u|.
 template <bool XS, class Team>
 __device__ __noinline__ void eig_vectors(const Team tm, const float* d, const float* e, const float* lam, int n,
-                                         float* X, int ld, float* S, float* M, float* inorm) {
+                                         float* X, int ld, float2* SM, float* inorm) {
   EIG_SHARED(d);
   EIG_SHARED(e);
   EIG_SHARED(lam);
@@ -599,6 +592,7 @@ __device__ __noinline__ void eig_vectors(const Team tm, const float* d, const fl
   for (int u = tr; u < n; u += ts) {
     const float x = lam[u];
     float* Xu = X + u * ld;
+    float2* sm = SM + u;
     float a = d[0] - x, b = e[0];
     for (int i = 0; i + 1 < n; i += 4) {
       // rows i .. i + 3: d_{i+1..i+4}, e_{i..i+4} (zero beyond the end)
@@ -612,8 +606,7 @@ __device__ __noinline__ void eig_vectors(const Team tm, const float* d, const fl
           const bool swp = fabsf(a) < fabsf(ei);
           if (!swp && fabsf(a) < TINY) a = copysignf(TINY, a);
           const float mlt = __fdividef(swp ? a : ei, swp ? ei : a);
-          S[(i + k) * n + u] = a;
-          M[(i + k) * n + u] = mlt;
+          sm[(i + k) * n] = make_float2(a, mlt);
           a = fmaf(-mlt, swp ? dn : b, swp ? b : dn);
           b = swp ? -mlt * en : en;
         }
@@ -623,53 +616,60 @@ __device__ __noinline__ void eig_vectors(const Team tm, const float* d, const fl
     const float ial = __fdividef(1.f, a);
     float f = 1.f;
     for (int it = 0; it < 2; ++it) {
-      float r = 0.f;
+      float r = it ? Xu[0] * f : eig_noise(n - 1, u);
       if (it) {                                    // forward elimination of the first vector
-        r = Xu[0] * f;
+        float2 nx[AH];
+#pragma unroll
+        for (int k = 0; k < AH; ++k) nx[k] = sm[min(k, n - 1) * n];
         for (int i0 = 0; i0 + 1 < n; i0 += AH) {
-          float mv[AH], sv[AH], xv[AH];
+          float2 cu[AH];
+          float xv[AH], ev[AH];
 #pragma unroll
           for (int k = 0; k < AH; ++k) {
-            const int i = min(i0 + k, n - 2);
-            mv[k] = M[i * n + u];
-            sv[k] = S[i * n + u];
-            xv[k] = Xu[i + 1] * f;
+            cu[k] = nx[k];
+            xv[k] = Xu[min(i0 + k + 1, n - 1)] * f;
+            ev[k] = fabsf(e[min(i0 + k, n - 1)]);
           }
 #pragma unroll
+          for (int k = 0; k < AH; ++k) nx[k] = sm[min(i0 + AH + k, n - 1) * n];
+#pragma unroll
           for (int k = 0; k < AH; ++k) {
-            const int i = i0 + k;
-            if (i + 1 < n) {
-              const bool swp = fabsf(sv[k]) < fabsf(e[i]);
-              Xu[i] = swp ? xv[k] : r;
-              r = fmaf(-mv[k], swp ? xv[k] : r, swp ? r : xv[k]);
+            if (i0 + k + 1 < n) {
+              const bool swp = fabsf(cu[k].x) < ev[k];
+              Xu[i0 + k] = swp ? xv[k] : r;
+              r = fmaf(-cu[k].y, swp ? xv[k] : r, swp ? r : xv[k]);
             }
           }
         }
-      } else {
-        r = eig_noise(n - 1, u);
       }
       float x1 = r * ial, x2 = 0.f, nn = x1 * x1;
       Xu[n - 1] = x1;
+      // rows n - 2 .. 0; row i also needs the pivot and the multiplier of row i - 1
+      float2 nx[AH + 1];
+#pragma unroll
+      for (int k = 0; k <= AH; ++k) nx[k] = sm[max(n - 2 - k, 0) * n];
       for (int i0 = n - 2; i0 >= 0; i0 -= AH) {
-        float sv[AH + 1], mp[AH], yv[AH];
+        float2 cu[AH + 1];
+        float y[AH], iu0[AH], u1[AH], u2[AH];
 #pragma unroll
-        for (int k = 0; k < AH; ++k) {
+        for (int k = 0; k <= AH; ++k) cu[k] = nx[k];
+#pragma unroll
+        for (int k = 0; k <= AH; ++k) nx[k] = sm[max(i0 - AH - k, 0) * n];
+#pragma unroll
+        for (int k = 0; k < AH; ++k) {             // all that does not wait for the row before
           const int i = max(i0 - k, 0);
-          sv[k] = S[i * n + u];
-          mp[k] = M[max(i - 1, 0) * n + u];
-          yv[k] = it ? Xu[i] : eig_noise(i, u);
+          const float ei = e[i], en = e[i + 1], ep = e[max(i - 1, 0)], dn = d[i + 1] - x;
+          const bool swp = fabsf(cu[k].x) < fabsf(ei), swq = i > 0 && fabsf(cu[k + 1].x) < fabsf(ep);
+          y[k] = it ? Xu[i] : eig_noise(i, u);
+          iu0[k] = __fdividef(1.f, swp ? ei : cu[k].x);
+          u1[k] = swp ? dn : (swq ? -cu[k + 1].y * ei : ei);
+          u2[k] = swp ? en : 0.f;
         }
-        sv[AH] = S[max(i0 - AH, 0) * n + u];
 #pragma unroll
         for (int k = 0; k < AH; ++k) {
-          const int i = i0 - k;
-          if (i >= 0) {
-            const float ei = e[i], en = e[i + 1], ai = sv[k];
-            const bool swp = fabsf(ai) < fabsf(ei), swq = i > 0 && fabsf(sv[k + 1]) < fabsf(e[max(i - 1, 0)]);
-            const float bi = swq ? -mp[k] * ei : ei;
-            const float u0 = swp ? ei : ai, u1 = swp ? d[i + 1] - x : bi, u2 = swp ? en : 0.f;
-            const float xi = fmaf(-u1, x1, fmaf(-u2, x2, yv[k])) * __fdividef(1.f, u0);
-            Xu[i] = xi;
+          if (i0 - k >= 0) {
+            const float xi = fmaf(-u1[k], x1, fmaf(-u2[k], x2, y[k])) * iu0[k];
+            Xu[i0 - k] = xi;
             nn = fmaf(xi, xi, nn);
             x2 = x1;
             x1 = xi;
@@ -686,9 +686,10 @@ __device__ __noinline__ void eig_vectors(const Team tm, const float* d, const fl
 // X <- H_0 ... H_{n-3} X diag(inorm): a 4-lane group holds NV vectors in registers, each
 // lane NC chunks of four consecutive components (16 c + 4 lane ..).
 template <int NC, int NV, bool XS, class Team>
-__device__ __noinline__ void eig_back(const Team tm, const float* A, const float* tau, int n, float* X, int ld,
-                                      const float* inorm) {
+__device__ __noinline__ void eig_back(const Team tm, const float* A, const float* V0, const float* tau, int n, float* X,
+                                      int ld, const float* inorm) {
   EIG_SHARED(A);
+  EIG_SHARED(V0);
   EIG_SHARED(tau);
   EIG_SHARED(inorm);
   if (XS) EIG_SHARED(X);
@@ -710,11 +711,12 @@ __device__ __noinline__ void eig_back(const Team tm, const float* A, const float
     }
     for (int j = n - 3; j >= 0; --j) {
       const float t = tau[j];
-      const float* Aj = A + j * ld + 4 * gl;
+      const float* Aj = (j > 0 ? A + (j - 1) * ld : V0) + 4 * gl;   // reflector j
       float4 rv[NC];
+      float2 ds[NV];
       float dt[NV];
 #pragma unroll
-      for (int q = 0; q < NV; ++q) dt[q] = 0.f;
+      for (int q = 0; q < NV; ++q) ds[q] = make_float2(0.f, 0.f);
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
         rv[c] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -724,7 +726,10 @@ __device__ __noinline__ void eig_back(const Team tm, const float* A, const float
       for (int c = 0; c < NC; ++c)
 #pragma unroll
         for (int q = 0; q < NV; ++q)
-          dt[q] = fmaf(rv[c].x, z[q][c].x, fmaf(rv[c].y, z[q][c].y, fmaf(rv[c].z, z[q][c].z, fmaf(rv[c].w, z[q][c].w, dt[q]))));
+          ds[q] = ffma2(make_float2(rv[c].x, rv[c].y), make_float2(z[q][c].x, z[q][c].y),
+                        ffma2(make_float2(rv[c].z, rv[c].w), make_float2(z[q][c].z, z[q][c].w), ds[q]));
+#pragma unroll
+      for (int q = 0; q < NV; ++q) dt[q] = ds[q].x + ds[q].y;
 #pragma unroll
       for (int o = 2; o > 0; o >>= 1)
 #pragma unroll
@@ -732,12 +737,12 @@ __device__ __noinline__ void eig_back(const Team tm, const float* A, const float
 #pragma unroll
       for (int q = 0; q < NV; ++q) {
         const float g = -t * dt[q];
+        const float2 g2 = make_float2(g, g);
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
-          z[q][c].x = fmaf(g, rv[c].x, z[q][c].x);
-          z[q][c].y = fmaf(g, rv[c].y, z[q][c].y);
-          z[q][c].z = fmaf(g, rv[c].z, z[q][c].z);
-          z[q][c].w = fmaf(g, rv[c].w, z[q][c].w);
+          const float2 lo = ffma2(g2, make_float2(rv[c].x, rv[c].y), make_float2(z[q][c].x, z[q][c].y));
+          const float2 hi = ffma2(g2, make_float2(rv[c].z, rv[c].w), make_float2(z[q][c].z, z[q][c].w));
+          z[q][c] = make_float4(lo.x, lo.y, hi.x, hi.y);
         }
       }
     }
@@ -804,7 +809,7 @@ __device__ __noinline__ float eig_defect(const Team tm, const float* X, int n, i
     while (jq * (jq + 1) / 2 > t) --jq;
     while ((jq + 1) * (jq + 2) / 2 <= t) ++jq;
     const int iq = t - jq * (jq + 1) / 2;
-    float acc[4][4];
+    float2 acc[4][4];
     const float4* xi[4];
     const float4* xj[4];
 #pragma unroll
@@ -812,7 +817,7 @@ __device__ __noinline__ float eig_defect(const Team tm, const float* X, int n, i
       xi[a] = reinterpret_cast<const float4*>(X + min(4 * iq + a, n - 1) * ld);
       xj[a] = reinterpret_cast<const float4*>(X + min(4 * jq + a, n - 1) * ld);
 #pragma unroll
-      for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
+      for (int b = 0; b < 4; ++b) acc[a][b] = make_float2(0.f, 0.f);
     }
     for (int r = 0; r < nq; ++r) {
       float4 va[4], vb[4];
@@ -825,7 +830,8 @@ __device__ __noinline__ float eig_defect(const Team tm, const float* X, int n, i
       for (int a = 0; a < 4; ++a)
 #pragma unroll
         for (int b = 0; b < 4; ++b)
-          acc[a][b] = fmaf(va[a].x, vb[b].x, fmaf(va[a].y, vb[b].y, fmaf(va[a].z, vb[b].z, fmaf(va[a].w, vb[b].w, acc[a][b]))));
+          acc[a][b] = ffma2(make_float2(va[a].x, va[a].y), make_float2(vb[b].x, vb[b].y),
+                            ffma2(make_float2(va[a].z, va[a].w), make_float2(vb[b].z, vb[b].w), acc[a][b]));
     }
 #pragma unroll
     for (int a = 0; a < 4; ++a)
@@ -833,7 +839,7 @@ __device__ __noinline__ float eig_defect(const Team tm, const float* X, int n, i
       for (int b = 0; b < 4; ++b) {
         const int i = 4 * iq + a, j = 4 * jq + b;
         if (i < n && j < n && i <= j) {
-          const float v = (i == j ? 1.f : 0.f) - acc[a][b];
+          const float v = (i == j ? 1.f : 0.f) - (acc[a][b].x + acc[a][b].y);
           worst = (fabsf(v) <= worst) ? worst : fabsf(v);      // NaN stays
           E[i * ld + j] = v;
           E[j * ld + i] = v;
@@ -844,44 +850,57 @@ __device__ __noinline__ float eig_defect(const Team tm, const float* X, int n, i
   worst = fminf(worst, 1e30f);
   return tm.max(worst);                            // ends with a team barrier
 }
-// out (row stride lo) = X + E X / 2 over the vectors
+// out (row stride lo = ld) = X + E X / 2 over the vectors
 template <bool XS, class Team>
 __device__ __noinline__ void eig_correct(const Team tm, const float* X, const float* E, int n, int ld, float* out, int lo) {
   EIG_SHARED(E);
   if (XS) EIG_SHARED(X);
   const int tr = tm.rank(), ts = tm.size();
-  const int nq = (n + 3) >> 2;
-  for (int t = tr; t < nq * nq; t += ts) {
-    const int iq = t / nq, jq = t % nq;            // vectors 4 iq.., components 4 jq..
-    float acc[4][4];
+  const int nq = (n + 3) >> 2, nc = lo >> 2;
+  for (int t = tr; t < nq * nc; t += ts) {
+    const int iq = t / nc, jq = t % nc;            // vectors 4 iq.., components 4 jq.. (pad components zero)
+    float2 acc[4][2];
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
+    for (int a = 0; a < 4; ++a) acc[a][0] = acc[a][1] = make_float2(0.f, 0.f);
 #pragma unroll 4
     for (int k = 0; k < n; ++k) {
       const float4 x = *reinterpret_cast<const float4*>(X + k * ld + 4 * jq);
       const float4 y = *reinterpret_cast<const float4*>(E + k * ld + 4 * iq);
-      const float xa[4] = {x.x, x.y, x.z, x.w}, ya[4] = {y.x, y.y, y.z, y.w};
+      const float2 x0 = make_float2(x.x, x.y), x1 = make_float2(x.z, x.w);
+      const float ya[4] = {y.x, y.y, y.z, y.w};
 #pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(ya[a], xa[b], acc[a][b]);
+      for (int a = 0; a < 4; ++a) {
+        const float2 y2 = make_float2(ya[a], ya[a]);
+        acc[a][0] = ffma2(y2, x0, acc[a][0]);
+        acc[a][1] = ffma2(y2, x1, acc[a][1]);
+      }
     }
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const int i = 4 * iq + a, j = 4 * jq + b;
-        if (i < n && j < n) out[i * lo + j] = fmaf(0.5f, acc[a][b], X[i * ld + j]);
+    for (int a = 0; a < 4; ++a) {
+      const int i = 4 * iq + a;
+      if (i < n) {
+        const float4 x = *reinterpret_cast<const float4*>(X + i * ld + 4 * jq);   // pad components are zero
+        *reinterpret_cast<float4*>(out + i * lo + 4 * jq) =
+            make_float4(fmaf(0.5f, acc[a][0].x, x.x), fmaf(0.5f, acc[a][0].y, x.y), fmaf(0.5f, acc[a][1].x, x.z),
+                        fmaf(0.5f, acc[a][1].y, x.w));
       }
+    }
   }
+  tm.sync();
+}
+// 16-byte copies, `words` a multiple of 4 and both sides aligned
+template <class Team>
+__device__ __forceinline__ void eig_copy(const Team& tm, const float* from, int words, float* to) {
+  const float4* f = reinterpret_cast<const float4*>(from);
+  float4* t = reinterpret_cast<float4*>(to);
+#pragma unroll 4
+  for (int x = tm.rank(); x < words / 4; x += tm.size()) t[x] = f[x];
   tm.sync();
 }
 
 template <bool XS, class Team>
 __device__ int eig_start_at(const Team tm, const uint4* At, int m, int n, float* A, float* X, float* V, float* Xg,
-                            float* lamg, float* Sg) {
+                            float* lamg, float2* Sg) {
   const int tr = tm.rank(), ts = tm.size();
   const int ld = eig_ld(n);
   float* W = V + 2 * ld;
@@ -895,11 +914,11 @@ __device__ int eig_start_at(const Team tm, const uint4* At, int m, int n, float*
   eig_tridiag(tm, A, n, ld, V, W, P, d, e, tau, inorm + ld);
   const float sc = eig_values(tm, d, e, n, ld, reinterpret_cast<float2*>(P), lam);
   for (int x = tr; x < n * (ld - n); x += ts) X[(x / (ld - n)) * ld + n + x % (ld - n)] = 0.f;
-  eig_vectors<XS>(tm, d, e, lam, n, X, ld, Sg, Xg, inorm);   // Xg is free until the vectors are finished
-  if (n <= 16) eig_back<1, 2, XS>(tm, A, tau, n, X, ld, inorm);
-  else if (n <= 48) eig_back<3, 2, XS>(tm, A, tau, n, X, ld, inorm);
-  else if (n <= 80) eig_back<5, 2, XS>(tm, A, tau, n, X, ld, inorm);
-  else eig_back<EIG_MAXN / 16, 1, XS>(tm, A, tau, n, X, ld, inorm);
+  eig_vectors<XS>(tm, d, e, lam, n, X, ld, Sg, inorm);
+  if (n <= 16) eig_back<1, 2, XS>(tm, A, V, tau, n, X, ld, inorm);
+  else if (n <= 48) eig_back<3, 2, XS>(tm, A, V, tau, n, X, ld, inorm);
+  else if (n <= 80) eig_back<5, 2, XS>(tm, A, V, tau, n, X, ld, inorm);
+  else eig_back<EIG_MAXN / 16, 1, XS>(tm, A, V, tau, n, X, ld, inorm);
   eig_clusters<XS>(tm, lam, n, X, ld);
   const float isc = __fdividef(1.f, sc);
   for (int u = tr; u < n; u += ts) lamg[u] = fmaxf(lam[u] * isc, 0.f);
@@ -908,22 +927,21 @@ __device__ int eig_start_at(const Team tm, const uint4* At, int m, int n, float*
   for (int it = 0; it < 10; ++it) {
     const float worst = eig_defect<XS>(tm, X, n, ld, A);
     if (!(worst < 1.5f)) return 3;
-    eig_correct<XS>(tm, X, A, n, ld, Xg, n);
+    eig_correct<XS>(tm, X, A, n, ld, Xg, ld);
     if (worst < 5e-4f) return 0;                   // the defect after the correction is its square
-    for (int x = tr; x < n * n; x += ts) X[(x / n) * ld + x % n] = Xg[x];
-    tm.sync();
+    eig_copy(tm, Xg, n * ld, X);
   }
   return 3;
 }
 // Approximate eigenvectors and eigenvalues of B^T B.  At: the digits of B^T (eig_digits); arena:
-// `words` floats of shared memory (16-byte aligned); Xg (n x n floats, row stride n, one
-// vector per row, eigenvalues descending) and lamg (n floats) receive the result, Sg (n x
-// n floats) and Xalt (n x ld floats, for X where the arena only holds A) are scratch, all
+// `words` floats of shared memory (16-byte aligned); Xg (n x ld floats, one vector per
+// row, pad components zero, eigenvalues descending) and lamg (n floats) receive the result, Sg (n x
+// n pairs) and Xalt (n x ld floats, for X where the arena only holds A) are scratch, all
 // in global memory.  Returns 0, 1 if the block does not fit (no result), or 3 if X is not
 // orthonormal in the end (the eigenvalues hold).
 template <class Team>
 __device__ int eig_start(const Team& tm, const uint4* At, int m, int n, float* arena, int words, float* Xg, float* lamg,
-                         float* Sg, float* Xalt) {
+                         float2* Sg, float* Xalt) {
   const int ld = eig_ld(n);
   if (n > EIG_MAXN || n * ld + eig_vec_floats(n) > words) return 1;
   if (2 * n * ld + eig_vec_floats(n) <= words)
@@ -944,8 +962,7 @@ __device__ __noinline__ void eig_bx(const Team tm, const uint4* A, const uint2* 
     float acc[NS - 1][4];
     mma_tile<NA, NB, NS>(A, D, it, j, KT, JT, lane, acc);
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-      W[(size_t)(8 * j + t2 + (q & 1)) * ldw + 16 * it + g + 8 * (q >> 1)] = mma_value<NS>(acc, q, 0);
+    for (int q = 0; q < 4; ++q) W[(8 * j + t2 + (q & 1)) * ldw + 16 * it + g + 8 * (q >> 1)] = mma_value<NS>(acc, q, 0);
   }
   tm.sync();
 }
@@ -961,7 +978,7 @@ __device__ __noinline__ void eig_residual(const Team tm, const uint4* At, const 
     const int it = t % nt, j = t / nt;
     float2 xv[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) xv[q] = Xd[(size_t)(8 * j + t2 + (q & 1)) * ldx + 16 * it + g + 8 * (q >> 1)];
+    for (int q = 0; q < 4; ++q) xv[q] = Xd[(8 * j + t2 + (q & 1)) * ldx + 16 * it + g + 8 * (q >> 1)];
     float acc[NS - 1][4];
     mma_tile<NA, NB, NS>(At, D, it, j, KT, JT, lane, acc);
 #pragma unroll
@@ -1011,8 +1028,9 @@ __device__ __noinline__ float eig_angles(const Team tm, const float* X, const fl
   for (int t = warp; t < rc * kcn; t += nw) {
     const int i = (t % rc) * 32 + lane, k0 = (t / rc) * EIG_TC;
     float s[EIG_TC];
+    float2 s2[EIG_TC];
 #pragma unroll
-    for (int q = 0; q < EIG_TC; ++q) s[q] = 0.f;
+    for (int q = 0; q < EIG_TC; ++q) s2[q] = make_float2(0.f, 0.f);
     const float4* xp = reinterpret_cast<const float4*>(X + min(i, n - 1) * ld);
     const float4* rp = reinterpret_cast<const float4*>(R + k0 * ld);
     const int l4 = ld >> 2;
@@ -1022,9 +1040,11 @@ __device__ __noinline__ float eig_angles(const Team tm, const float* X, const fl
 #pragma unroll
       for (int q = 0; q < EIG_TC; ++q) {
         const float4 r = rp[q * l4 + c];
-        s[q] = fmaf(x.x, r.x, fmaf(x.y, r.y, fmaf(x.z, r.z, fmaf(x.w, r.w, s[q]))));
+        s2[q] = ffma2(make_float2(x.x, x.y), make_float2(r.x, r.y), ffma2(make_float2(x.z, x.w), make_float2(r.z, r.w), s2[q]));
       }
     }
+#pragma unroll
+    for (int q = 0; q < EIG_TC; ++q) s[q] = s2[q].x + s2[q].y;
     if (i < n) {
       const float2 li = i < kc ? lk[i] : make_float2(lam[i], 0.f);
       float o[EIG_TC];
@@ -1050,7 +1070,7 @@ __device__ __noinline__ float eig_angles(const Team tm, const float* X, const fl
   if (!(worst >= 0.f)) worst = 1e30f;
   return tm.max(fminf(worst, 1e30f));
 }
-// Xd (column k at k ldx) += X^T T, and the FP32 vectors Xg (row k at k n) follow: lanes are components.
+// Xd (column k at k ldx) += X^T T, and the FP32 vectors Xg (row k at k ld) follow: lanes are components.
 template <class Team>
 __device__ __noinline__ void eig_update(const Team tm, const float* X, const float* T, int n, int ld, int kc, int kp,
                                         float2* Xd, int ldx, float* Xg) {
@@ -1059,45 +1079,42 @@ __device__ __noinline__ void eig_update(const Team tm, const float* X, const flo
   const int rc = (n + 31) >> 5, kcn = kp / EIG_TC;
   for (int t = warp; t < rc * kcn; t += nw) {
     const int i = (t % rc) * 32 + lane, k0 = (t / rc) * EIG_TC, ic = min(i, n - 1);
-    float s[EIG_TC];
+    float2 s2[EIG_TC / 2];
     float2 xv[EIG_TC];
 #pragma unroll
-    for (int q = 0; q < EIG_TC; ++q) {
-      s[q] = 0.f;
-      xv[q] = Xd[(size_t)(k0 + q) * ldx + ic];
-    }
+    for (int q = 0; q < EIG_TC; ++q) xv[q] = Xd[(size_t)(k0 + q) * ldx + ic];
+#pragma unroll
+    for (int q = 0; q < EIG_TC / 2; ++q) s2[q] = make_float2(0.f, 0.f);
     const float* xp = X + ic;
 #pragma unroll 4
     for (int v = 0; v < n; ++v) {
       const float x = xp[v * ld];
+      const float2 x2 = make_float2(x, x);
       const float4 ra = *reinterpret_cast<const float4*>(T + v * kp + k0);
       const float4 rb = *reinterpret_cast<const float4*>(T + v * kp + k0 + 4);
-      s[0] = fmaf(x, ra.x, s[0]);
-      s[1] = fmaf(x, ra.y, s[1]);
-      s[2] = fmaf(x, ra.z, s[2]);
-      s[3] = fmaf(x, ra.w, s[3]);
-      s[4] = fmaf(x, rb.x, s[4]);
-      s[5] = fmaf(x, rb.y, s[5]);
-      s[6] = fmaf(x, rb.z, s[6]);
-      s[7] = fmaf(x, rb.w, s[7]);
+      s2[0] = ffma2(x2, make_float2(ra.x, ra.y), s2[0]);
+      s2[1] = ffma2(x2, make_float2(ra.z, ra.w), s2[1]);
+      s2[2] = ffma2(x2, make_float2(rb.x, rb.y), s2[2]);
+      s2[3] = ffma2(x2, make_float2(rb.z, rb.w), s2[3]);
     }
+    const float s[EIG_TC] = {s2[0].x, s2[0].y, s2[1].x, s2[1].y, s2[2].x, s2[2].y, s2[3].x, s2[3].y};
     if (i < n) {
 #pragma unroll
       for (int q = 0; q < EIG_TC; ++q) {
         const float2 v = dfa::add(xv[q], make_float2(s[q], 0.f));
         Xd[(size_t)(k0 + q) * ldx + i] = v;
-        if (k0 + q < kc) Xg[(k0 + q) * n + i] = v.x;
+        if (k0 + q < kc) Xg[(k0 + q) * ld + i] = v.x;
       }
     }
   }
   tm.sync();
 }
 
-// Refines the first kc vectors of Xg (n x n, one per row; updated) as described at the top.  A, At: the
+// Refines the first kc vectors of Xg (n x ld, one per row; updated) as described at the top.  A, At: the
 // digits of B and B^T; lam0 the approximate eigenvalues.  Outputs: Wout (column j at j m), Qout
 // (column j at j n) in FP64, the singular values in sig[0..kc).  Wd, Xd (kp columns of length m
 // and n padded to 16, double-floats), Dg (digits of either) and Xalt (n x ld floats) are global
-// scratch; the last two are used where the arena is too small.  Returns 0, or 1 if the
+// scratch, used where the arena is too small.  Returns 0, or 1 if the
 // corrections do not converge or the block does not fit.
 template <class Team>
 __device__ int eig_refine(const Team& tm, const uint4* A, const uint4* At, int m, int n, int kc, float* Xg,
@@ -1116,9 +1133,16 @@ __device__ int eig_refine(const Team& tm, const uint4* A, const uint4* At, int m
   uint2* D = fix + dig <= words ? reinterpret_cast<uint2*>(T) : Dg;
   const bool xin = fix + tx + n * ld <= words;
   float* X = xin ? T + tx : Xalt;
+  // what is left behind the larger of the two takes the columns themselves
+  int at = fix + max(fix + dig <= words ? dig : 0, tx + (xin ? n * ld : 0));
+  if (at + 2 * n16 * kp <= words) {
+    Xd = reinterpret_cast<float2*>(arena + at);
+    at += 2 * n16 * kp;
+  }
+  if (at + 2 * m16 * kp <= words) Wd = reinterpret_cast<float2*>(arena + at);
   for (int x = tr; x < n16 * kp; x += ts) {
     const int k = x / n16, c = x % n16;
-    float v = (k < kc && c < n) ? Xg[k * n + c] : 0.f;
+    float v = (k < kc && c < n) ? Xg[k * ld + c] : 0.f;
     // four digits carry the start vectors: entries below 2^-7 are rounded to 2^-30
     if (fabsf(v) < 0.0078125f) v = __fsub_rn(__fadd_rn(v, 0.01171875f), 0.01171875f);
     Xd[x] = make_float2(v, 0.f);
@@ -1147,11 +1171,7 @@ __device__ int eig_refine(const Team& tm, const uint4* A, const uint4* At, int m
       eig_digits_cols<EIG_DIG>(tm, Wd, m16, m, kp, EIG_WEXP, D);
       eig_residual<EIG_DIG, EIG_DIG, EIG_DIG + 1>(tm, At, D, m, n, kp, Xd, n16, lk, R, ld);
     }
-    for (int x = tr; x < n * ld; x += ts) {
-      const int u = x / ld, c = x % ld;
-      X[x] = c < n ? Xg[u * n + c] : 0.f;
-    }
-    tm.sync();
+    eig_copy(tm, Xg, n * ld, X);
     const float worst = eig_angles(tm, X, R, n, ld, kc, kp, lk, ek, lam, T);
     if (!(worst < 0.05f)) return 1;
     eig_update(tm, X, T, n, ld, kc, kp, Xd, n16, Xg);
