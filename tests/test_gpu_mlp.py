@@ -78,3 +78,24 @@ def test_training_reduces_loss():
             net.adam_step(X, T, lr=3e-3)
         l1 = net.gradient(X, T)[0]
     assert l1 < 0.05 * l0
+
+
+@pytest.mark.parametrize("n_in,n_h,n_out,B", [(1, 1, 1, 1), (31, 33, 32, 65), (65, 32, 1, 63), (33, 64, 31, 129),
+                                              (5, 300, 7, 700)])
+def test_tile_edges_match_oracle(n_in, n_h, n_out, B):
+    """Sizes around the 32-wide tiles and slabs and the cuts of the batch (64 rows and up).  Sums have at most
+    700 terms: 700 x 6e-8 of their absolute terms, so 1e-4 of a tensor's largest entry as above."""
+    net, flat, X, T, w = setup(n_in, n_h, n_out, B, seed=n_in + B)
+    with net:
+        p = om.unpack(flat.astype(np.float64), n_in, n_h, n_out)
+        X64, T64 = X.astype(np.float64), T.astype(np.float64)
+        Yo, _ = om.forward(p, X64)
+        assert np.abs(net.forward(X) - Yo).max() <= 1e-5 * max(1.0, np.abs(Yo).max())
+        for ww in (w, None):
+            L, g = net.gradient(X, T, ww)
+            Lo, go = om.gradient(p, X64, T64, None if ww is None else ww.astype(np.float64))
+            assert abs(L - Lo) <= 1e-5 * abs(Lo)
+            a = om.unpack(g.astype(np.float64), n_in, n_h, n_out)
+            for name in om.NAMES:
+                assert np.abs(a[name] - go[name]).max() <= 1e-4 * np.abs(go[name]).max(), name
+            assert net.last_launches() == 7
