@@ -95,6 +95,24 @@ def test_decay_to_the_cutoff_keeps_what_is_above_it(n):
     assert np.abs(Bn.reshape(k, -1) @ Bn.reshape(k, -1).T - np.eye(k)).max() <= 2e-12
 
 
+@pytest.mark.parametrize("n", [2, 4, 5, 8, 9])
+@pytest.mark.parametrize("low", [1e-13, 1e-17, 1e-20, 1e-40])
+def test_columns_of_very_different_lengths_converge(n, low):
+    """Columns from 1 down to far below the rounding of the longest (their order and signs mixed), as a product of
+    decaying bonds leaves them: the SVD ends and keeps what is above the cutoff."""
+    rng = np.random.default_rng(n)
+    d = 10.0 ** np.linspace(0.0, np.log10(low), n)[rng.permutation(n)]
+    A, B, qL, qM, qR = one_block(n + 2, n, np.ones(n), rng)
+    A[:, 3, :] = rng.normal(size=(n + 2, n)) * d
+    B[:, 3, :] = np.eye(n)
+    An, Bn, k, disc = gate(A, B, qL, qM, qR, 0, n, 1e-14)
+    m = A[:, 3, :]
+    new = np.tensordot(An, Bn, axes=([2], [0]))[:, 3, 3, :]
+    # backward stable in the 2-norm: m n eps of the largest, plus what the cutoff drops
+    assert np.linalg.norm(new - m) <= (4.0 * U48 * n + 1e-14 * n) * np.linalg.norm(m)
+    assert np.abs(Bn.reshape(k, -1) @ Bn.reshape(k, -1).T - np.eye(k)).max() <= 2e-12
+
+
 @pytest.mark.parametrize("n,rank", [(6, 6), (20, 20), (40, 17), (64, 30), (64, 64)])
 def test_degenerate_and_rank_deficient_blocks_are_kept_whole(n, rank):
     rng = np.random.default_rng(n + rank)
