@@ -19,9 +19,13 @@
 //        x <- x + X t,  t_i = X_i . r / (lambda - lambda_i),  t_k = (1 - |x|^2) / 2
 //      (Ogita and Aishima, Japan J. Indust. Appl. Math. 35 (2018) 1007, with the
 //      residual formed before the projection, so that the products with X and
-//      the update only need FP32).  It converges quadratically: on the gates of
-//      N = 14, chi = 128 states |t| is at most 1e-4, then 1e-8, then at rounding
-//      level, so two corrections.
+//      the update only need FP32).  It converges quadratically in the kept vectors and
+//      by 1e-6 over the relative distance of the eigenvalues along the dropped ones,
+//      whose eigenvalues stay FP32: on the gates of N = 14, chi = 128 states |t| is at
+//      most 1e-4, then 1e-8, so two corrections, sometimes three.  Last, the kept
+//      vectors are orthonormalised by their inner products (I + (I - X^T X) / 2): the
+//      corrections alone leave 1e-13, and the matrix elements ten times the rounding
+//      error of an FP64 SVD.
 // Whatever this cannot do (a kept singular value below 5e-3 of the block's
 // largest one, a cluster that leaves X dependent, a correction that does not
 // shrink) is reported, and the caller takes the one-sided Jacobi SVD.
@@ -46,10 +50,12 @@ namespace {
 
 constexpr int EIG_NE = 5;                          // lanes' share of a row: n <= 32 EIG_NE
 constexpr int EIG_MAXN = 32 * EIG_NE;
+// A correction below this is the last.  (1e-8 leaves errors of 5e-16 in overlaps of N = 12, chi = 64 states with
+// decaying spectra where an FP64 SVD and 1e-9 leave 1e-16; rotation of N = 14, chi = 128 83 against 87 ms.)
+constexpr float EIG_ACCEPT = 1e-9f;
 constexpr float EIG_MIN_LAMBDA = 3e-5f;            // kept lambda over the block's largest: sigma ratio 5.5e-3
 constexpr int EIG_TC = 8;                          // kept columns per task (an mma's n)
 constexpr int EIG_DIG = 7;                         // digits of an operand
-constexpr int EIG_WEXP = 4;                        // |w| < 2^(1 + EIG_WEXP): 2 sqrt(256)
 
 __device__ __forceinline__ float warp_sum_f(float v) {
 #pragma unroll
@@ -201,14 +207,16 @@ __device__ __noinline__ void eig_digits(const Team tm, const double* raw, int m,
 }
 
 // B-operand fragments of the columns k = 0..kp-1 of V (column k at k ldv, double-floats, |entries| <
-// 2^(1 + ex), length K padded with zeros to a multiple of 16): the 16 x 8 tile (kt, jt) has its digits
-// at ((kt JT + jt) ND + s) 32 + lane.
+// 2^(1 + exs[k]), exs null: 2; length K padded with zeros to a multiple of 16): the 16 x 8 tile (kt, jt)
+// has its digits at ((kt JT + jt) ND + s) 32 + lane.
 template <int ND, class Team>
-__device__ __noinline__ void eig_digits_cols(const Team tm, const float2* V, int ldv, int K, int kp, int ex, uint2* D) {
+__device__ __noinline__ void eig_digits_cols(const Team tm, const float2* V, int ldv, int K, int kp, const int* exs,
+                                             uint2* D) {
   const int lane = threadIdx.x & 31, warp = tm.rank() >> 5, nw = tm.size() >> 5;
   const int kt = pad16(K) >> 4, jt = kp >> 3, g = lane >> 2, t2 = 2 * (lane & 3);
   for (int t = warp; t < kt * jt; t += nw) {
     const int k = t / jt, j = t % jt;
+    const int ex = exs ? exs[8 * j + g] : 0;
     const float4* p = reinterpret_cast<const float4*>(V + (size_t)(8 * j + g) * ldv + 16 * k + t2);
     const float4 lo = p[0], hi = p[4];
     unsigned a[EIG_DIG], b[EIG_DIG];
@@ -966,10 +974,11 @@ __device__ __noinline__ void eig_bx(const Team tm, const uint4* A, const uint2* 
   }
   tm.sync();
 }
-// R (column k at k ld) = B^T W - X lambda from the digits of B^T (At) and of W (D).
+// R (column k at k ld) = B^T W - X lambda from the digits of B^T (At) and of W (D, scaled by 2^-exs[k]).
 template <int NA, int NB, int NS, class Team>
 __device__ __noinline__ void eig_residual(const Team tm, const uint4* At, const uint2* D, int m, int n, int kp,
-                                          const float2* Xd, int ldx, const float2* lk, float* R, int ld) {
+                                          const float2* Xd, int ldx, const float2* lk, const int* exs, float* R,
+                                          int ld) {
   EIG_SHARED(lk);
   EIG_SHARED(R);
   const int lane = threadIdx.x & 31, warp = tm.rank() >> 5, nw = tm.size() >> 5;
@@ -985,7 +994,7 @@ __device__ __noinline__ void eig_residual(const Team tm, const uint4* At, const 
     for (int q = 0; q < 4; ++q) {
       const int k = 8 * j + t2 + (q & 1), c = 16 * it + g + 8 * (q >> 1);
       const float2 lx = dfa::mul(lk[k], xv[q]);
-      const float2 df = dfa::add(mma_value<NS>(acc, q, EIG_WEXP), make_float2(-lx.x, -lx.y));
+      const float2 df = dfa::add(mma_value<NS>(acc, q, exs[k]), make_float2(-lx.x, -lx.y));
       if (c < ld) R[k * ld + c] = c < n ? df.x + df.y : 0.f;
     }
   }
@@ -1013,7 +1022,9 @@ __device__ __forceinline__ void eig_norms(const Team& tm, const float2* V, int l
   }
 }
 // T (row i at i kp) = X R / (lambda_k - lambda_i), half the norm's defect ek on the diagonal: lanes are
-// vectors i.  Returns the largest |entry|.
+// vectors i.  lam: the eigenvalues of the discarded vectors, FP32 (1e-6 lam[0] or better): a correction leaves
+// 1e-6 lam[0] / |lambda_k - lambda_i| of itself along those.  Returns the largest |entry|, along
+// discarded vectors closer than 1e-3 lam[0] times 1e-3 lam[0] / |lambda_k - lambda_i|.
 template <class Team>
 __device__ __noinline__ float eig_angles(const Team tm, const float* X, const float* R, int n, int ld, int kc, int kp,
                                          const float2* lk, const float* ek, const float* lam, float* T) {
@@ -1047,19 +1058,22 @@ __device__ __noinline__ float eig_angles(const Team tm, const float* X, const fl
     for (int q = 0; q < EIG_TC; ++q) s[q] = s2[q].x + s2[q].y;
     if (i < n) {
       const float2 li = i < kc ? lk[i] : make_float2(lam[i], 0.f);
+      const float near = i < kc ? 0.f : 1e-3f * lam[0];
       float o[EIG_TC];
 #pragma unroll
       for (int q = 0; q < EIG_TC; ++q) {
         const int k = k0 + q;
-        float v = 0.f;
+        float v = 0.f, w = 1.f;
         if (k < kc) {
           if (i == k) {
             v = 0.5f * ek[k];
           } else {
             const float den = (lk[k].x - li.x) + (lk[k].y - li.y);
             v = den != 0.f ? __fdividef(s[q], den) : (s[q] == 0.f ? 0.f : 1e30f);
+            if (fabsf(den) < near) w = __fdividef(near, fabsf(den));
           }
-          worst = (fabsf(v) <= worst) ? worst : fabsf(v);
+          w *= fabsf(v);
+          worst = (w <= worst) ? worst : w;
         }
         o[q] = v;
       }
@@ -1070,10 +1084,42 @@ __device__ __noinline__ float eig_angles(const Team tm, const float* X, const fl
   if (!(worst >= 0.f)) worst = 1e30f;
   return tm.max(fminf(worst, 1e30f));
 }
-// Xd (column k at k ldx) += X^T T, and the FP32 vectors Xg (row k at k ld) follow: lanes are components.
+// T (row i at i kp, kc rows) = half the defect of the kept vectors' inner products, (I - X^T X) / 2: eight
+// lanes per pair.
 template <class Team>
-__device__ __noinline__ void eig_update(const Team tm, const float* X, const float* T, int n, int ld, int kc, int kp,
-                                        float2* Xd, int ldx, float* Xg) {
+__device__ __noinline__ void eig_orth(const Team tm, const float2* Xd, int ldx, int n, int kc, int kp, float* T) {
+  EIG_SHARED(T);
+  const int gl = tm.rank() & 7, ng = tm.size() >> 3, np = kc * (kc + 1) / 2;
+  for (int x = tm.rank(); x < kc * kp; x += tm.size()) T[x] = 0.f;   // (columns beyond kc)
+  tm.sync();
+  for (int p0 = 0; p0 < np; p0 += ng) {
+    const int p = min(p0 + (tm.rank() >> 3), np - 1);
+    const float f = 8.f * (float)p + 1.f;
+    int k = (int)((f * rsqrtf(f) - 1.f) * 0.5f);
+    while (k * (k + 1) / 2 > p) --k;
+    while ((k + 2) * (k + 1) / 2 <= p) ++k;
+    const int i = p - k * (k + 1) / 2;
+    const float2* a = Xd + (size_t)i * ldx;
+    const float2* b = Xd + (size_t)k * ldx;
+    float s = 0.f, er = 0.f;
+#pragma unroll 2
+    for (int r = gl; r < n; r += 8) dot2_step(a[r], b[r], s, er);
+    float2 l = df_pair(s, er);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1)
+      l = dfa::add(l, make_float2(__shfl_xor_sync(0xffffffffu, l.x, o), __shfl_xor_sync(0xffffffffu, l.y, o)));
+    if (gl == 0) {
+      const float e = 0.5f * __fadd_rn(__fadd_rn(i == k ? 1.f : 0.f, -l.x), -l.y);
+      T[i * kp + k] = e;
+      T[k * kp + i] = e;
+    }
+  }
+  tm.sync();
+}
+// Xd (column k at k ldx) += X^T T (nv rows), and the FP32 vectors Xg (row k at k ld) follow: lanes are components.
+template <class Team>
+__device__ __noinline__ void eig_update(const Team tm, const float* X, const float* T, int nv, int n, int ld, int kc,
+                                        int kp, float2* Xd, int ldx, float* Xg) {
   EIG_SHARED(T);
   const int lane = threadIdx.x & 31, warp = tm.rank() >> 5, nw = tm.size() >> 5;
   const int rc = (n + 31) >> 5, kcn = kp / EIG_TC;
@@ -1087,7 +1133,7 @@ __device__ __noinline__ void eig_update(const Team tm, const float* X, const flo
     for (int q = 0; q < EIG_TC / 2; ++q) s2[q] = make_float2(0.f, 0.f);
     const float* xp = X + ic;
 #pragma unroll 4
-    for (int v = 0; v < n; ++v) {
+    for (int v = 0; v < nv; ++v) {
       const float x = xp[v * ld];
       const float2 x2 = make_float2(x, x);
       const float4 ra = *reinterpret_cast<const float4*>(T + v * kp + k0);
@@ -1122,12 +1168,14 @@ __device__ int eig_refine(const Team& tm, const uint4* A, const uint4* At, int m
                           double* Wout, double* Qout, double* sig, double scale) {
   const int tr = tm.rank(), ts = tm.size();
   const int ld = eig_ld(n), kp = eig_kp(kc), m16 = pad16(m), n16 = pad16(n);
-  // arena: lk (kp float2), ek (kp), lam (ld), R (kp x ld), then the digits or, after them, T (n x kp) and X (n x ld)
-  const int fix = 3 * kp + ld + kp * ld, dig = m16 * kp * EIG_DIG / 2, tx = n * kp;
+  // arena: lk (kp float2), ek and exs (kp), lam (ld), R (kp x ld), then the digits or, after them, T
+  // (n x kp) and X (n x ld)
+  const int fix = 4 * kp + ld + kp * ld, dig = m16 * kp * EIG_DIG / 2, tx = n * kp;
   if (fix + tx > words) return 1;
   float2* lk = reinterpret_cast<float2*>(arena);
   float* ek = arena + 2 * kp;
-  float* lam = ek + kp;
+  int* exs = reinterpret_cast<int*>(ek + kp);
+  float* lam = ek + 2 * kp;
   float* R = lam + ld;
   float* T = R + kp * ld;
   uint2* D = fix + dig <= words ? reinterpret_cast<uint2*>(T) : Dg;
@@ -1152,33 +1200,38 @@ __device__ int eig_refine(const Team& tm, const uint4* A, const uint4* At, int m
   for (int it = 0; it < 6; ++it) {
     // the first correction starts from 1e-6 and needs 1e-10: six digits of B, four of X
     if (it == 0) {
-      eig_digits_cols<4>(tm, Xd, n16, n, kp, 0, D);
+      eig_digits_cols<4>(tm, Xd, n16, n, kp, nullptr, D);
       eig_bx<6, 4, 7>(tm, A, D, m, n, kp, Wd, m16);
     } else {
-      eig_digits_cols<EIG_DIG>(tm, Xd, n16, n, kp, 0, D);
+      eig_digits_cols<EIG_DIG>(tm, Xd, n16, n, kp, nullptr, D);
       eig_bx<EIG_DIG, EIG_DIG, EIG_DIG + 1>(tm, A, D, m, n, kp, Wd, m16);
     }
     eig_norms(tm, Wd, m16, m, kp, [&](int k, float2 l) {
       lk[k] = l;
-      if (k < kc) lam[k] = l.x;
+      exs[k] = (((__float_as_int(l.x) >> 23) & 255) - 127) >> 1;     // |w| < 2^(1 + exs)
     });
     eig_norms(tm, Xd, n16, n, kp, [&](int k, float2 l) { ek[k] = __fadd_rn(__fadd_rn(1.f, -l.x), -l.y); });
     tm.sync();
     if (it == 0) {
-      eig_digits_cols<6>(tm, Wd, m16, m, kp, EIG_WEXP, D);
-      eig_residual<6, 6, 7>(tm, At, D, m, n, kp, Xd, n16, lk, R, ld);
+      eig_digits_cols<6>(tm, Wd, m16, m, kp, exs, D);
+      eig_residual<6, 6, 7>(tm, At, D, m, n, kp, Xd, n16, lk, exs, R, ld);
     } else {
-      eig_digits_cols<EIG_DIG>(tm, Wd, m16, m, kp, EIG_WEXP, D);
-      eig_residual<EIG_DIG, EIG_DIG, EIG_DIG + 1>(tm, At, D, m, n, kp, Xd, n16, lk, R, ld);
+      eig_digits_cols<EIG_DIG>(tm, Wd, m16, m, kp, exs, D);
+      eig_residual<EIG_DIG, EIG_DIG, EIG_DIG + 1>(tm, At, D, m, n, kp, Xd, n16, lk, exs, R, ld);
     }
     eig_copy(tm, Xg, n * ld, X);
     const float worst = eig_angles(tm, X, R, n, ld, kc, kp, lk, ek, lam, T);
-    if (!(worst < 0.05f)) return 1;
-    eig_update(tm, X, T, n, ld, kc, kp, Xd, n16, Xg);
-    if (worst <= 1e-8f) break;
+    if (!(worst < 0.25f)) return 1;
+    eig_update(tm, X, T, n, n, ld, kc, kp, Xd, n16, Xg);
+    if (worst <= EIG_ACCEPT) break;
     if (it == 5) return 1;
   }
-  eig_digits_cols<EIG_DIG>(tm, Xd, n16, n, kp, 0, D);
+  // The kept vectors orthonormal to the working precision: what is left of the corrections' products, and the
+  // rounding of R over the differences of the eigenvalues, which differs in T_ik and T_ki.
+  eig_orth(tm, Xd, n16, n, kc, kp, T);
+  eig_copy(tm, Xg, kc * ld, X);
+  eig_update(tm, X, T, kc, n, ld, kc, kp, Xd, n16, Xg);
+  eig_digits_cols<EIG_DIG>(tm, Xd, n16, n, kp, nullptr, D);
   eig_bx<EIG_DIG, EIG_DIG, EIG_DIG + 1>(tm, A, D, m, n, kp, Wd, m16);
   eig_norms(tm, Wd, m16, m, kp, [&](int k, float2 l) {
     if (k < kc) sig[k] = sqrt(dfa::to_double(l)) * scale;

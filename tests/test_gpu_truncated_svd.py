@@ -113,6 +113,29 @@ def test_columns_of_very_different_lengths_converge(n, low):
     assert np.abs(Bn.reshape(k, -1) @ Bn.reshape(k, -1).T - np.eye(k)).max() <= 2e-12
 
 
+@pytest.mark.parametrize("n", [12, 30, 60, 90])
+@pytest.mark.parametrize("close", [1e-3, 1e-6, 1e-9, 1e-12])
+def test_close_singular_values_at_the_cut_keep_the_vectors_orthonormal(n, close):
+    """Eight singular values within `close` of one another around the cut, down to where the approximate vectors mix
+    kept and dropped ones and the refinement gives up."""
+    rng = np.random.default_rng(n)
+    k = n // 2
+    sg = np.linspace(1.0, 0.05, n)
+    sg[k - 4: k + 4] = sg[k] * (1.0 + close * np.linspace(1.0, -1.0, 8))
+    A, B, qL, qM, qR = one_block(n + 1, n, sg, rng)
+    An, Bn, kn, disc = gate(A, B, qL, qM, qR, 0, k, 1e-12)
+    th = np.tensordot(A, B, axes=([2], [0])).reshape((n + 1) * 4, -1)
+    new = np.tensordot(An, Bn, axes=([2], [0])).reshape(th.shape)
+    assert kn == k
+    # double-float vectors and products (sums of n terms)
+    V = Bn.reshape(k, -1)
+    assert np.abs(V @ V.T - np.eye(k)).max() <= 4.0 * U48 * np.sqrt(n)
+    assert np.abs(th @ V.T - An.reshape(-1, k)).max() <= 4.0 * U48 * np.sqrt(n)
+    # any k-dimensional choice among the close ones drops the same weight up to close^2 of it
+    best = float((sg[k:] ** 2).sum())
+    assert np.linalg.norm(new - th) ** 2 <= best * (1.0 + 1e-10 + 8.0 * close) and disc <= best * (1.0 + 1e-10 + 8.0 * close)
+
+
 @pytest.mark.parametrize("n,rank", [(6, 6), (20, 20), (40, 17), (64, 30), (64, 64)])
 def test_degenerate_and_rank_deficient_blocks_are_kept_whole(n, rank):
     rng = np.random.default_rng(n + rank)
