@@ -1840,18 +1840,17 @@ void check_ctx(tnqe_ctx* c) {
 // particle-number block structure, (n_alpha, n_beta) sector, left-orthonormal
 // sites 0..N-2), sort every bond by charge and lay the tensors out in that
 // order (host, back to back; offsets in m.off).  Throws Error(TNQE_ERR_ARG).
-// Run f(0..n-1) on up to 8 host threads (static interleaved shares).
-template <class F> void parallel_for(int n, F f) {
-  const int nt = std::max(1, std::min({n, 8, (int)std::thread::hardware_concurrency()}));
-  if (nt <= 1) {
-    for (int i = 0; i < n; ++i) f(i);
-    return;
-  }
+// Run f(0..n-1) on up to 8 host threads, the caller's among them (static interleaved shares): one for every
+// 64 K of the `work` entries to visit (about 50 us of a pass; starting a thread costs 20 to 40).
+template <class F> void parallel_for(int n, long long work, F f) {
+  const int nt = (int)std::max(1LL, std::min({(long long)n, 8LL, (long long)std::thread::hardware_concurrency(),
+                                              work / 65536}));
   std::vector<std::thread> th;
-  for (int t = 0; t < nt; ++t)
+  for (int t = 1; t < nt; ++t)
     th.emplace_back([&, t]() {
       for (int i = t; i < n; i += nt) f(i);
     });
+  for (int i = 0; i < n; i += nt) f(i);
   for (auto& x : th) x.join();
 }
 
@@ -1887,12 +1886,18 @@ void order_mps_host(int N, int na, int nb, const double* const* tensors, const i
   std::vector<double> amax(N, 0.0);
   for (int s = 0; s < N; ++s)
     if (!tensors[s]) throw Error(TNQE_ERR_ARG, "null site tensor");
-  parallel_for(N, [&](int s) {
+  long long entries = 0;
+  for (int s = 0; s < N; ++s) entries += (long long)bond_dims[s] * 4 * bond_dims[s + 1];
+  parallel_for(N, entries, [&](int s) {
     const double* A = tensors[s];
     const long long n = (long long)bond_dims[s] * 4 * bond_dims[s + 1];
-    double mx = 0.0;
-    for (long long x = 0; x < n; ++x) mx = std::max(mx, std::fabs(A[x]));
-    amax[s] = mx;
+    double mx[4] = {0.0, 0.0, 0.0, 0.0};           // four chains
+    for (long long x = 0; x < n; x += 4)           // n is a multiple of 4
+      for (int h = 0; h < 4; ++h) {
+        const double v = std::fabs(A[x + h]);
+        mx[h] = v > mx[h] ? v : mx[h];
+      }
+    amax[s] = std::max(std::max(mx[0], mx[1]), std::max(mx[2], mx[3]));
   });
   std::vector<std::vector<int>> q(N + 1);
   q[0] = {0};
@@ -1918,29 +1923,40 @@ void order_mps_host(int N, int na, int nb, const double* const* tensors, const i
       break;
     }
   }
-  // the block-structure checks of the sites whose charges are known (all of
-  // them unless a bond index has no weight), then the errors in site order
-  const int nok = noweight >= 0 ? noweight : N;
-  std::vector<int> bad_block(N, 0);
-  parallel_for(nok, [&](int s) {
-    const int cl = bond_dims[s], cr = bond_dims[s + 1];
-    const double* A = tensors[s];
-    const double tol = 1e-12 * amax[s];
-    const std::vector<int>& qr0 = q[s + 1];
-    for (int l = 0; l < cl && !bad_block[s]; ++l)
-      for (int k = 0; k < 4; ++k) {
-        const int qlk = (q[s][l] / QSTRIDE + (k & 1)) * QSTRIDE + q[s][l] % QSTRIDE + (k >> 1);
-        const double* row = A + ((size_t)l * 4 + k) * cr;
-        for (int r = 0; r < cr; ++r)
-          if (std::fabs(row[r]) > tol && qr0[r] != qlk) bad_block[s] = 1;
-      }
-  });
-  for (int s = 0; s < nok; ++s)
-    if (bad_block[s])
-      throw Error(TNQE_ERR_ARG, "site " + std::to_string(s) + ": entry breaks the particle-number block structure");
-  if (noweight >= 0)
+  // Errors come in this order: entries outside the blocks (by site), an index without weight, the sector, the
+  // number of charges, orthonormality.  The first check is part of the pass that writes the sites (every
+  // pass over the entries costs memory time); where a later error is known already, it runs alone.
+  std::vector<int> bad_block(N, 0), bad_orth(N, 0);
+  auto row_bad = [&](int s, const double* row, int qlk, double tol) {
+    const int* qr0 = q[s + 1].data();
+    int bad = 0;
+    for (int r = 0, cr = bond_dims[s + 1]; r < cr; ++r) bad |= (int)(std::fabs(row[r]) > tol) & (int)(qr0[r] != qlk);
+    return bad;
+  };
+  auto row_charge = [&](int s, int l, int k) {
+    return (q[s][l] / QSTRIDE + (k & 1)) * QSTRIDE + q[s][l] % QSTRIDE + (k >> 1);
+  };
+  auto block_error = [&](int upto) {
+    for (int s = 0; s < upto; ++s)
+      if (bad_block[s])
+        throw Error(TNQE_ERR_ARG, "site " + std::to_string(s) + ": entry breaks the particle-number block structure");
+  };
+  auto check_blocks = [&](int upto) {
+    parallel_for(upto, entries, [&](int s) {
+      for (int lk = 0; lk < bond_dims[s] * 4 && !bad_block[s]; ++lk)
+        bad_block[s] = row_bad(s, tensors[s] + (size_t)lk * bond_dims[s + 1], row_charge(s, lk >> 2, lk & 3),
+                               1e-12 * amax[s]);
+    });
+    block_error(upto);
+  };
+  if (noweight >= 0) {
+    check_blocks(noweight);
     throw Error(TNQE_ERR_ARG, "site " + std::to_string(noweight) + ": bond index with no weight");
-  if (q[N][0] != na * QSTRIDE + nb) throw Error(TNQE_ERR_ARG, "state is not in the (n_alpha, n_beta) sector");
+  }
+  if (q[N][0] != na * QSTRIDE + nb) {
+    check_blocks(N);
+    throw Error(TNQE_ERR_ARG, "state is not in the (n_alpha, n_beta) sector");
+  }
   // sort every bond by charge (a gauge change: the state is unchanged)
   std::vector<std::vector<int>> perm(N + 1);
   m.dims.assign(bond_dims, bond_dims + N + 1);
@@ -1955,7 +1971,10 @@ void order_mps_host(int N, int na, int nb, const double* const* tensors, const i
     for (int x = 0; x < bond_dims[b]; ++x) {
       const int qq = q[b][perm[b][x]];
       if (T.nsec == 0 || T.q[T.nsec - 1] != qq) {
-        if (T.nsec >= MAXSEC) throw Error(TNQE_ERR_ARG, "too many charge sectors on one bond");
+        if (T.nsec >= MAXSEC) {
+          check_blocks(N);
+          throw Error(TNQE_ERR_ARG, "too many charge sectors on one bond");
+        }
         T.q[T.nsec] = qq;
         T.off[T.nsec] = x;
         T.dim[T.nsec] = 0;
@@ -1972,47 +1991,45 @@ void order_mps_host(int N, int na, int nb, const double* const* tensors, const i
   }
   out.n = total;
   if (!(out.ext && out.ext_cap >= total)) out.p.reset(new double[total]);   // every entry is written below
-  // one pass per site, sites on host threads: sites 0..N-2 left-orthonormal (the Gram matrix of the
-  // columns, block by block: columns of different charge have disjoint support);
-  // the site written in the sorted order, zero outside the blocks
-  std::vector<int> bad_orth(N, 0);
-  parallel_for(N, [&](int s) {
+  // one pass per site, sites on host threads: the block check; the site written in the sorted order, zero
+  // outside the blocks; sites 0..N-2 left-orthonormal (the Gram matrix of the columns of every charge, from
+  // the sorted rows: columns of different charge have disjoint support)
+  parallel_for(N, entries, [&](int s) {
     const int cl = bond_dims[s], cr = bond_dims[s + 1];
     const double* A = tensors[s];
-    const std::vector<int>& qr0 = q[s + 1];
-    if (s + 1 < N) {
-      std::vector<double> gram((size_t)cr * cr, 0.0);
-      std::vector<std::vector<int>> same(cr);      // columns of r's charge at or after r
-      for (int r1 = 0; r1 < cr; ++r1)
-        for (int r2 = r1; r2 < cr; ++r2)
-          if (qr0[r1] == qr0[r2]) same[r1].push_back(r2);
-      for (int lk = 0; lk < cl * 4; ++lk) {
-        const double* row = A + (size_t)lk * cr;
-        for (int r1 = 0; r1 < cr; ++r1) {
-          const double a1 = row[r1];
-          if (a1 == 0.0) continue;
-          double* g = gram.data() + (size_t)r1 * cr;
-          for (int r2 : same[r1]) g[r2] += a1 * row[r2];
-        }
-      }
-      for (int r1 = 0; r1 < cr && !bad_orth[s]; ++r1)
-        for (int r2 : same[r1])
-          if (std::fabs(gram[(size_t)r1 * cr + r2] - (r1 == r2 ? 1.0 : 0.0)) > 1e-10) bad_orth[s] = 1;
-    }
-    std::vector<int> qr(cr);
-    for (int r = 0; r < cr; ++r) qr[r] = qr0[perm[s + 1][r]];
+    const double tol = 1e-12 * amax[s];
+    const SectorTable& T = m.sec[s + 1];
     const int* pr = perm[s + 1].data();
+    std::vector<int> goff(T.nsec + 1, 0);
+    for (int x = 0; x < T.nsec; ++x) goff[x + 1] = goff[x] + T.dim[x] * T.dim[x];
+    std::vector<double> gram(s + 1 < N ? goff[T.nsec] : 0, 0.0);
     double* dst0 = out.data() + m.off[s];
-    for (int l = 0; l < cl; ++l) {
-      const int ql = q[s][perm[s][l]];
+    for (int l = 0; l < cl; ++l)
       for (int k = 0; k < 4; ++k) {
-        const int qlk = (ql / QSTRIDE + (k & 1)) * QSTRIDE + ql % QSTRIDE + (k >> 1);
-        const double* src = A + ((size_t)perm[s][l] * 4 + k) * cr;
+        const int l0 = perm[s][l], qlk = row_charge(s, l0, k);
+        const double* src = A + ((size_t)l0 * 4 + k) * cr;
         double* dst = dst0 + ((size_t)l * 4 + k) * cr;
-        for (int r = 0; r < cr; ++r) dst[r] = (qlk == qr[r]) ? src[pr[r]] : 0.0;   // below-tolerance noise outside the blocks
+        bad_block[s] |= row_bad(s, src, qlk, tol);
+        int x = 0;
+        while (x < T.nsec && T.q[x] != qlk) ++x;
+        const int o = x < T.nsec ? T.off[x] : 0, d = x < T.nsec ? T.dim[x] : 0;
+        std::fill(dst, dst + o, 0.0);                // also below-tolerance noise outside the blocks
+        for (int r = o; r < o + d; ++r) dst[r] = src[pr[r]];
+        std::fill(dst + o + d, dst + cr, 0.0);
+        if (s + 1 < N)
+          for (int a = 0; a < d; ++a) {
+            const double v = dst[o + a];
+            if (v == 0.0) continue;
+            double* g = gram.data() + goff[x] + (size_t)a * d;
+            for (int b = a; b < d; ++b) g[b] += v * dst[o + b];
+          }
       }
-    }
+    for (int x = 0; x < T.nsec && s + 1 < N; ++x)
+      for (int a = 0; a < T.dim[x]; ++a)
+        for (int b = a; b < T.dim[x]; ++b)
+          if (std::fabs(gram[goff[x] + (size_t)a * T.dim[x] + b] - (a == b ? 1.0 : 0.0)) > 1e-10) bad_orth[s] = 1;
   });
+  block_error(N);
   for (int s = 0; s + 1 < N; ++s)
     if (bad_orth[s]) throw Error(TNQE_ERR_ARG, "site " + std::to_string(s) + " is not left-orthonormal");
 }

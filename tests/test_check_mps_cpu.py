@@ -93,3 +93,35 @@ def test_states_of_the_benchmark_workload_are_valid():
     w = inputs.workload("n14_chi128")
     for m in w.mps[:4]:
         assert tnqe.tnqe_check_mps(m.tensors, m.U, w.n_alpha, w.n_beta) == (0, "")
+
+
+@pytest.mark.parametrize("chi", [5, 48, 100])
+def test_checks_of_unsorted_bonds_on_one_and_several_threads(chi):
+    """Bonds whose charges are not sorted, 0.05 to 0.5 M entries (one thread and several): a valid state passes, and
+    at every site an entry outside the blocks, a column without unit norm and two equal columns are found; an
+    entry outside the blocks comes before a wrong sector."""
+    w = inputs.make_workload(9, 4, 5, 4, 2, [chi], seed=chi, shuffle_bonds=True)
+    m, U = w.mps[1], w.mps[1].U
+    check = lambda ts, na=w.n_alpha: tnqe.tnqe_check_mps(ts, U, na, w.n_beta)
+    assert check(m.tensors) == (0, "")
+    for s in range(len(m.tensors)):
+        ts = [t.copy() for t in m.tensors]
+        zero = np.argwhere(ts[s] == 0.0)
+        if len(zero):
+            ts[s][tuple(zero[len(zero) // 2])] = 1e-3
+            st, msg = check(ts)
+            assert st == 1 and "block structure" in msg and f"site {s}" in msg
+            st, msg = check(ts, w.n_alpha - 1)
+            assert st == 1 and "block structure" in msg and f"site {s}" in msg
+        if s + 1 < len(m.tensors):
+            r = ts[s].shape[2] - 1
+            ts = [t.copy() for t in m.tensors]
+            ts[s][:, :, r] *= 1.0 + 1e-9
+            st, msg = check(ts)
+            assert st == 1 and "left-orthonormal" in msg and f"site {s}" in msg
+            same = [c for c in range(r) if m.charges[s + 1][c] == m.charges[s + 1][r]]
+            if same:
+                ts = [t.copy() for t in m.tensors]
+                ts[s][:, :, same[0]] = ts[s][:, :, r]
+                st, msg = check(ts)
+                assert st == 1 and "left-orthonormal" in msg and f"site {s}" in msg
