@@ -917,6 +917,7 @@ void run_contractions_bs(tnqe_ctx* c, const std::vector<std::pair<int, int>>& pa
     size_t base, od, op1, op2, op3, oe, of;
     int nw;
     std::vector<long long> tot1, tot2, tot3;
+    std::vector<int> chi;                          // largest bond at the site
   };
   std::vector<WaveLayout> lay(waves.size());
   std::vector<unsigned char> host;
@@ -946,6 +947,7 @@ void run_contractions_bs(tnqe_ctx* c, const std::vector<std::pair<int, int>>& pa
     L.tot1.resize(N);
     L.tot2.resize(N);
     L.tot3.resize(N);
+    L.chi.assign(N, 1);
     for (int t = 0; t < N; ++t) {
       long long n1 = 0, n2 = 0, n3 = 0;
       for (int w = 0; w < nw; ++w) {
@@ -975,6 +977,7 @@ void run_contractions_bs(tnqe_ctx* c, const std::vector<std::pair<int, int>>& pa
         d.chL = bi.bs_ch[t];
         d.chR = bi.bs_ch[t + 1];
         d.rows = bi.bs_rows[t];
+        L.chi[t] = std::max({L.chi[t], d.ca, d.ca2, d.capb, d.capb2});
         pre1.push_back(n1);
         pre2.push_back(n2);
         pre3.push_back(n3);
@@ -1025,13 +1028,13 @@ void run_contractions_bs(tnqe_ctx* c, const std::vector<std::pair<int, int>>& pa
       cudaEvent_t* E = &c->pev[e];
       record_event(c, E[0]);
       CKL(launch_bs_stage1(dsd + (size_t)t * nw, reinterpret_cast<const long long*>(dd + L.op1) + pofs, nw,
-                           L.tot1[t], dfl, c->tune.bs_t1, c->stream));
+                           L.tot1[t], L.chi[t], dfl, c->tune.bs_t1, c->stream));
       record_event(c, E[1]);
       CKL(launch_bs_stage2(dsd + (size_t)t * nw, reinterpret_cast<const long long*>(dd + L.op2) + pofs, nw,
-                           L.tot2[t], dfl, c->tune.bs_t2, c->stream));
+                           L.tot2[t], L.chi[t], dfl, c->tune.bs_t2, c->stream));
       record_event(c, E[2]);
       CKL(launch_bs_stage3(dsd + (size_t)t * nw, reinterpret_cast<const long long*>(dd + L.op3) + pofs, nw,
-                           L.tot3[t], dfl, c->tune.bs_t3, c->stream));
+                           L.tot3[t], L.chi[t], dfl, c->tune.bs_t3, c->stream));
       record_event(c, E[3]);
       c->launches += 3;
       reads.push_back({e, e + 1, 1});

@@ -9,9 +9,10 @@
 //   Y[a][k][w'][b']   != 0 only if q(b') = q(a) + q(k) - d(w')
 // (a nonzero W[(k, w'), (w, k')] has d(w') = d(w) + q(k) - q(k')).  The three
 // stages below compute and read exactly those blocks:
-//   stage 1  X = L B   one CTA per (pair, bra sector alpha of bond t, channel class c)
-//   stage 2  Y = W X   one CTA per (pair, bra index a); MPO rows grouped by d(w') - q(k)
-//   stage 3  L' = A^T Y one CTA per (pair, bra sector alpha' of bond t+1, channel class c')
+//   stage 1  X = L B   one item per (pair, bra sector alpha of bond t, channel class c)
+//   stage 2  Y = W X   one item per (pair, bra index a); MPO rows grouped by d(w') - q(k)
+//   stage 3  L' = A^T Y one item per (pair, bra sector alpha' of bond t+1, channel class c')
+// with one CTA per item, or up to eight where there are few.
 // The arrays keep the dense capacity layout, so nothing here depends on the
 // ket's sector dimensions except the sector tables the kernels read on the
 // device (for a rotated ket, the ones the rotation kernel wrote).  The small
@@ -20,12 +21,18 @@
 // operand loads (shared memory, L1) keeps the FP64 pipe the bound.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "internal.h"
 
 namespace tnqe {
 namespace {
 
-constexpr int BS_SMEM = 6144;                 // doubles of staged operand per CTA (48 KiB)
+// Doubles of staged operand per CTA (24 KiB): nine CTAs of 128 threads share an SM, so that staging, barriers
+// and the ragged ends of the small blocks of some hide behind the FP64 work of the others.  48 KiB (four
+// CTAs): stage 1 of N = 14, chi = 128 23.1 against 19.7 ms, stage 3 17.5 against 14.4; 16 KiB 19.7 and
+// 14.9 (operands in more pieces).
+constexpr int BS_SMEM = 3072;
 
 __device__ __forceinline__ int bs_problem(const long long* prefix, int n, long long x) {
   int lo = 0, hi = n - 1;
@@ -102,11 +109,13 @@ __global__ void __launch_bounds__(BS_THREADS) bs_stage1_kernel(const BsSiteDesc*
     return (((size_t)a * Din + w) * 4 + k) * capb2 + s_goff[k] + (j - s_gcol[k]);
   };
   if (dimB == 0) {
-    for (int o = tid; o < nrows * ncol; o += BS_THREADS) Xo[xaddr(o / ncol, o % ncol)] = 0.0;
+    for (int o = tid + BS_THREADS * blockIdx.y; o < nrows * ncol; o += BS_THREADS * gridDim.y)
+      Xo[xaddr(o / ncol, o % ncol)] = 0.0;
     return;
   }
-  if (tid == 0) atomicAdd(flops, 2.0 * nrows * dimB * ncol);
+  if (tid == 0 && blockIdx.y == 0) atomicAdd(flops, 2.0 * nrows * dimB * ncol);
   const int JC = min(ncol, BS_SMEM / dimB);
+  if (nrows * JC <= BS_THREADS * (int)blockIdx.y) return;
   for (int j0 = 0; j0 < ncol; j0 += JC) {
     const int jn = min(JC, ncol - j0);
     for (int x = tid; x < dimB * jn; x += BS_THREADS) {
@@ -115,7 +124,7 @@ __global__ void __launch_bounds__(BS_THREADS) bs_stage1_kernel(const BsSiteDesc*
       Bs[x] = Bt[((size_t)(offB + b) * 4 + k) * capb2 + s_goff[k] + (j - s_gcol[k])];
     }
     __syncthreads();
-    for (int o = tid; o < nrows * jn; o += BS_THREADS) {
+    for (int o = tid + BS_THREADS * blockIdx.y; o < nrows * jn; o += BS_THREADS * gridDim.y) {
       const int r = o / jn, jj = o % jn;
       const int a = offA + r / Dc, w = wl[r % Dc];
       const double* Lr = Lin + ((size_t)a * Din + w) * capb + offB;
@@ -159,7 +168,7 @@ __global__ void __launch_bounds__(BS_THREADS) bs_stage2_kernel(const BsSiteDesc*
     if (ig >= 0) atomicAdd(&s_fl, 2.0 * D.rows.nnz[r] * s_gdim[r]);
   }
   __syncthreads();
-  if (tid == 0 && s_fl > 0.0) atomicAdd(flops + 1, s_fl);
+  if (tid == 0 && blockIdx.y == 0 && s_fl > 0.0) atomicAdd(flops + 1, s_fl);
   const int capb2 = D.capb2;
   const double* __restrict__ Xa = D.X + (size_t)a * 4 * D.Din * capb2;
   double* __restrict__ Ya = D.Y + (size_t)a * 4 * D.Dout * capb2;
@@ -173,7 +182,7 @@ __global__ void __launch_bounds__(BS_THREADS) bs_stage2_kernel(const BsSiteDesc*
     if (dg == 0) continue;
     const int go = s_goff[r];
     const int r0 = roff[r], nr = roff[r + 1] - r0;
-    for (int o = tid; o < nr * dg; o += BS_THREADS) {
+    for (int o = tid + BS_THREADS * blockIdx.y; o < nr * dg; o += BS_THREADS * gridDim.y) {
       const int row = rrows[r0 + o / dg], g = go + o % dg;
       double acc = 0.0;
       const int e1 = rowptr[row + 1];
@@ -229,14 +238,15 @@ __global__ void __launch_bounds__(BS_THREADS) bs_stage3_kernel(const BsSiteDesc*
   const double* __restrict__ At = D.A;
   double* __restrict__ Lo = D.Lout;
   if (Kdim == 0) {
-    for (int o = tid; o < dimA2 * ncol; o += BS_THREADS) {
+    for (int o = tid + BS_THREADS * blockIdx.y; o < dimA2 * ncol; o += BS_THREADS * gridDim.y) {
       const int ap = o / ncol, j = o % ncol;
       Lo[((size_t)(offA2 + ap) * Dout + wl[j / dimB2]) * capb2 + offB2 + j % dimB2] = 0.0;
     }
     return;
   }
-  if (tid == 0) atomicAdd(flops + 2, 2.0 * dimA2 * ncol * Kdim);
+  if (tid == 0 && blockIdx.y == 0) atomicAdd(flops + 2, 2.0 * dimA2 * ncol * Kdim);
   const int AC = min(dimA2, BS_SMEM / Kdim);
+  if (((AC + 3) >> 2) * ncol <= BS_THREADS * (int)blockIdx.y) return;
   for (int a0 = 0; a0 < dimA2; a0 += AC) {
     const int an = min(AC, dimA2 - a0);
     for (int x = tid; x < Kdim * an; x += BS_THREADS) {
@@ -247,7 +257,7 @@ __global__ void __launch_bounds__(BS_THREADS) bs_stage3_kernel(const BsSiteDesc*
     }
     __syncthreads();
     const int ngrp = (an + 3) >> 2;
-    for (int o = tid; o < ngrp * ncol; o += BS_THREADS) {
+    for (int o = tid + BS_THREADS * blockIdx.y; o < ngrp * ncol; o += BS_THREADS * gridDim.y) {
       const int j = o % ncol, grp = o / ncol;
       const int wp = wl[j / dimB2], g = offB2 + j % dimB2;
       double acc[4] = {0.0, 0.0, 0.0, 0.0};
@@ -270,32 +280,44 @@ __global__ void __launch_bounds__(BS_THREADS) bs_stage3_kernel(const BsSiteDesc*
   }
 }
 
+// CTAs that share one item (bra sector x channel class, or bra index; every CTA stages the item's operand and
+// takes every y-th group of outputs).  The largest item of a site (the middle sectors times the class of the
+// neutral channels) is a fifth of a pair's work, so with few pairs one CTA was the time of the launch: N = 20,
+// chi = 128, one row of 8 pairs, stages 14.4 + 13.9 + 7.8 ms with one CTA per item, 5.0 + 8.7 + 3.6 with up to
+// eight.  No more than bring the launch to 20,000 CTAs (40,000 costs N = 14, chi = 128, 120 pairs 0.5 ms of
+// 61, 12,000 the row 2 of 17) and, where an operand is staged, one per 24 of the bond: small items do not fill
+// the CTAs (N = 10, chi = 32: 0.30 ms of stage 1 against 0.48 with eight).
+unsigned bs_split(long long total, int most) {
+  return (unsigned)std::max(1LL, std::min({20000 / total, (long long)most, 8LL}));
+}
+
 }  // namespace
 
-// CTA sizes of the stages (launch shapes the autotuner chooses from)
-#define BS_LAUNCH(kernel)                                                                                   \
+// CTA sizes of the stages (launch shapes the autotuner chooses from), `total` items on `y` CTAs each
+#define BS_LAUNCH(kernel, most)                                                                             \
   do {                                                                                                      \
     if (total <= 0) return 0;                                                                               \
     cudaStream_t st = (cudaStream_t)stream;                                                                 \
-    if (threads == 64) kernel<64><<<(unsigned)total, 64, 0, st>>>(d, prefix, n, flops);                     \
-    else if (threads == 256) kernel<256><<<(unsigned)total, 256, 0, st>>>(d, prefix, n, flops);             \
-    else kernel<128><<<(unsigned)total, 128, 0, st>>>(d, prefix, n, flops);                                 \
+    const dim3 grid((unsigned)total, bs_split(total, most));                                                 \
+    if (threads == 64) kernel<64><<<grid, 64, 0, st>>>(d, prefix, n, flops);                                \
+    else if (threads == 256) kernel<256><<<grid, 256, 0, st>>>(d, prefix, n, flops);                        \
+    else kernel<128><<<grid, 128, 0, st>>>(d, prefix, n, flops);                                            \
     return (int)cudaGetLastError();                                                                         \
   } while (0)
 
-int launch_bs_stage1(const BsSiteDesc* d, const long long* prefix, int n, long long total, double* flops,
+int launch_bs_stage1(const BsSiteDesc* d, const long long* prefix, int n, long long total, int chi, double* flops,
                      int threads, void* stream) {
-  BS_LAUNCH(bs_stage1_kernel);
+  BS_LAUNCH(bs_stage1_kernel, chi / 24);
 }
 
-int launch_bs_stage2(const BsSiteDesc* d, const long long* prefix, int n, long long total, double* flops,
+int launch_bs_stage2(const BsSiteDesc* d, const long long* prefix, int n, long long total, int chi, double* flops,
                      int threads, void* stream) {
-  BS_LAUNCH(bs_stage2_kernel);
+  BS_LAUNCH(bs_stage2_kernel, 8);
 }
 
-int launch_bs_stage3(const BsSiteDesc* d, const long long* prefix, int n, long long total, double* flops,
+int launch_bs_stage3(const BsSiteDesc* d, const long long* prefix, int n, long long total, int chi, double* flops,
                      int threads, void* stream) {
-  BS_LAUNCH(bs_stage3_kernel);
+  BS_LAUNCH(bs_stage3_kernel, chi / 24);
 }
 
 }  // namespace tnqe

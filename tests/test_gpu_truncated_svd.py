@@ -195,3 +195,16 @@ def test_solve_sizes_match_lapack(M):
     assert np.abs(E - ref).max() <= 64 * 2.2e-16 * M * np.abs(H).sum(0).max()
     assert np.abs(C.T @ S @ C - np.eye(M)).max() <= 64 * 2.2e-16 * M * np.abs(S).sum(0).max()
     assert np.abs(C.T @ H @ C - np.diag(E)).max() <= 64 * 2.2e-16 * M * np.abs(H).sum(0).max()
+
+
+@pytest.mark.parametrize("chi", [[30, 47], [48, 71], [100, 72, 97]])
+def test_contraction_items_shared_by_ctas_give_the_same_bits(chi):
+    """Few pairs (up to eight CTAs per item of a contraction stage, one per 24 of the bond) and many (one)."""
+    w = inputs.make_workload(8, 4, 4, 6, 3, chi, seed=7)
+    with tnqe.Context(w.h1, w.eri, w.N, w.n_alpha, w.n_beta) as g:
+        for m in w.mps:
+            g.add_mps(m.tensors, m.U)
+        base = [(i, j) for i in range(3) for j in range(3)]
+        H1, S1 = g.matrix_elements(base)
+        H2, S2 = g.matrix_elements(base * 30)
+    assert np.array_equal(np.tile(H1, 30), H2) and np.array_equal(np.tile(S1, 30), S2)
