@@ -347,11 +347,14 @@ __device__ __forceinline__ void df_fma_fused(float vh, float vl, float xh, float
 // memory once (each X element is read by every nonzero of its column).  The
 // slab arrives by cp.async, 16 bytes per copy where the rows allow it, so a
 // CTA keeps its whole slab in flight instead of one element per thread.  Each
-// thread then owns one row and all BW columns: BW independent double-float
+// thread then owns one row and BW / TPR columns: independent double-float
 // accumulations share every (value, column) load, and rows go in descending
-// nonzero count so the threads of a warp run loops of similar length.
+// nonzero count so the threads of a warp run loops of similar length.  The chain
+// of a long row (load, gather, ten dependent additions) is the time, so 512
+// threads and two CTAs per SM: 2.82 -> 2.31 ms for the own-basis energies of eight
+// N = 12, chi = 64 states against 256 threads (768: 2.68, 1024: 2.94 with one CTA).
 constexpr int SPMM_SMEM_BYTES = 112 * 1024;
-constexpr int SPMM_THREADS = 256;
+constexpr int SPMM_THREADS = 512;
 template <int BW, int TPR>
 __global__ void __launch_bounds__(SPMM_THREADS, 2) spmm_df_smem_kernel(const SpmmDfDesc* __restrict__ descs,
                                                                     const long long* __restrict__ prefix, int nprob) {

@@ -20,7 +20,9 @@
 // K-elements x rows x S slices, 64-byte swizzle) and the tcgen05.mma
 // instructions; loads run ahead into the next tile, so its first stages land
 // while the current tile's epilogue runs; the four accumulators take 4 BN
-// columns of tensor memory; all four warps run the epilogue, 16 columns at a
+// columns of tensor memory; eight warps run the epilogue (the products of the
+// contraction are short, K = chi, so it is most of a tile's time; four warps: 2.42
+// against 2.01 ms for N = 12, chi = 64, eight own-basis energies), 8 columns at a
 // time through a small per-warp staging buffer for row-contiguous stores.
 #pragma once
 #include <cuda.h>
@@ -33,12 +35,14 @@ constexpr int OZ_BM = 128, OZ_BK = 32;                 // BK in BF16 elements (6
 constexpr int OZ_BN_MAX = 128;                         // N tile: 128 or 64 (chosen per GEMM by the tuner)
 constexpr int OZ_MAXS = 5;                             // slices per operand
 constexpr int OZ_MAXK = 1024;                          // exactness bound of acc0..acc2
-constexpr int OZ_THREADS = 128;
+constexpr int OZ_THREADS = 256;
 constexpr int OZ_SLICE_BYTES = OZ_BM * OZ_BK * 2;      // 8 KiB per slice tile
 constexpr int OZ_MAX_STAGES = 4;
 constexpr int OZ_STAGE_AREA = 196608;                  // pipeline stages: 2 S slice tiles each
 constexpr int OZ_SLD = 17;                             // staging row stride (float2): 16 columns + 1
-constexpr int OZ_STAGING_BYTES = 4 * 32 * OZ_SLD * 8;  // per-warp epilogue staging, 16 columns at a time
+constexpr int OZ_SLD8 = 9;                             // the same for 8 columns (8 warps)
+constexpr int OZ_STAGING_BYTES = 8 * 32 * OZ_SLD8 * 8; // per-warp epilogue staging
+static_assert(OZ_STAGING_BYTES >= 4 * 32 * OZ_SLD * 8, "4 warps of 16 columns fit too");
 constexpr int OZ_SMEM_BYTES = OZ_STAGE_AREA + OZ_STAGING_BYTES + 1024 /*align*/ + 256 /*barriers*/;
 // bytes of one pipeline stage: S slice tiles of A (128 rows) and of B (BN rows)
 __host__ __device__ constexpr int oz_stage_bytes(int S, int BN) { return S * (OZ_SLICE_BYTES + BN * OZ_BK * 2); }
@@ -172,7 +176,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   using namespace ozdev;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  float2* staging = reinterpret_cast<float2*>(smem + OZ_STAGE_AREA);          // 4 warps x 32 rows x OZ_SLD
+  float2* staging = reinterpret_cast<float2*>(smem + OZ_STAGE_AREA);          // 8 warps x 32 rows x OZ_SLD8
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + OZ_STAGE_AREA + OZ_STAGING_BYTES);
   uint64_t* empty = full + OZ_MAX_STAGES;
   uint64_t* accb = empty + OZ_MAX_STAGES;
@@ -296,7 +300,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     }
     if (warp != 0)
       for (int i = tid - 32; i < BN; i += OZ_THREADS - 32) s_eb[i] = me.n0 + i < me.d->N ? me.d->eb[me.n0 + i] : 0;
-    const int row = me.m0 + warp * 32 + lane;
+    const int wrow = (warp & 3) * 32;                   // the warp's rows of the tile; its columns: half warp >> 2
+    const int row = me.m0 + wrow + lane;
     const int era = row < me.d->M ? me.d->ea[row] : 0;
     if (!mbar_wait(accb, (uint32_t)(ntile & 1), max_spin)) fail = 1;
     tc_fence_after();
@@ -306,14 +311,15 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     if (s_fail) break;
     // ---- epilogue: TMEM -> (hi, lo) -> per-warp staging -> rows of C
     {
-      const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
-      float2* stg = staging + warp * 32 * OZ_SLD;
+      const uint32_t lane_base = tmem + ((uint32_t)wrow << 16);
+      float2* stg = staging + warp * 32 * OZ_SLD8;
       const int ncols = min(BN, me.d->N - me.n0);
       const int mrows = me.d->M;
       const long long ldc = me.d->ldc;
       float2* Ct = me.d->C + me.n0;
+      const int cend = min(ncols, (warp >> 2) * (BN / 2) + BN / 2);
 #pragma unroll 1
-      for (int c0 = 0; c0 < BN; c0 += 16) {
+      for (int c0 = (warp >> 2) * (BN / 2); c0 < cend; c0 += 16) {
         uint32_t v0[16], v1[16], v2[16], v3[16];
         tmem_ld16(lane_base + 0 * BN + c0, v0);
         tmem_ld16(lane_base + 1 * BN + c0, v1);
@@ -321,27 +327,31 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         tmem_ld16(lane_base + 3 * BN + c0, v3);
         tmem_wait_ld();
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          float s, e, e2;
-          two_sum(__uint_as_float(v0[j]), __uint_as_float(v1[j]), s, e);
-          two_sum(s, __uint_as_float(v2[j]), s, e2);
-          e += e2;
-          if (S >= 3) e += __uint_as_float(v3[j]);
-          const float h = s + e;
-          const float l = e - (h - s);
-          const int ex = era + s_eb[c0 + j];
-          const float s1 = pow2f(ex / 2), s2 = pow2f(ex - ex / 2);
-          stg[lane * OZ_SLD + j] = make_float2(h * s1 * s2, l * s1 * s2);
+        for (int h = 0; h < 2; ++h) {                 // 8 columns at a time through the staging buffer
+#pragma unroll
+          for (int jj = 0; jj < 8; ++jj) {
+            const int j = 8 * h + jj;
+            float s, e, e2;
+            two_sum(__uint_as_float(v0[j]), __uint_as_float(v1[j]), s, e);
+            two_sum(s, __uint_as_float(v2[j]), s, e2);
+            e += e2;
+            if (S >= 3) e += __uint_as_float(v3[j]);
+            const float hi = s + e;
+            const float lo = e - (hi - s);
+            const int ex = era + s_eb[c0 + j];
+            const float s1 = pow2f(ex / 2), s2 = pow2f(ex - ex / 2);
+            stg[lane * OZ_SLD8 + jj] = make_float2(hi * s1 * s2, lo * s1 * s2);
+          }
+          __syncwarp();
+          const int col = c0 + 8 * h + (lane & 7);
+#pragma unroll
+          for (int rr = 0; rr < 32; rr += 4) {
+            const int r = rr + (lane >> 3);
+            const int grow = me.m0 + wrow + r;
+            if (grow < mrows && col < ncols) Ct[(long long)grow * ldc + col] = stg[r * OZ_SLD8 + (lane & 7)];
+          }
+          __syncwarp();
         }
-        __syncwarp();
-        const int col = c0 + (lane & 15);
-#pragma unroll 4
-        for (int rr = 0; rr < 32; rr += 2) {
-          const int r = rr + (lane >> 4);
-          const int grow = me.m0 + warp * 32 + r;
-          if (grow < mrows && col < ncols) Ct[(long long)grow * ldc + col] = stg[r * OZ_SLD + (lane & 15)];
-        }
-        __syncwarp();
       }
     }
     tc_fence_before();
