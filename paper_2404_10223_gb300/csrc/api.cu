@@ -853,8 +853,7 @@ void run_contractions(tnqe_ctx* c, const std::vector<std::pair<int, int>>& pairs
 // ----------------------------------------------------------------------------- block-sparse FP64 contraction
 // The dense form's workspace and layout, with only the charge-allowed blocks
 // computed (kernels_block.cu).  Work items per site: stage 1 and stage 3 one
-// CTA per (pair, bra sector, channel class), stage 2 one CTA per (pair, bra
-// index).  Algorithmic FLOPs are counted on the device (the ket's sector
+// per (pair, bra sector, channel class), stage 2 one per (pair, bra index).  Algorithmic FLOPs are counted on the device (the ket's sector
 // dimensions are decided there) and read back when the call has finished.
 // Profiling events of site t of workspace wave w: wave 0 uses the context's
 // per-site slots, later waves slots appended after the slicing events.

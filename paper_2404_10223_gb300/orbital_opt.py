@@ -10,7 +10,7 @@ and in its permutation-only variant accepts an FSWAP (the theta = pi/2 Givens
 gate up to a phase) when it lowers xi.
 
 Each evaluation of xi(theta) is one call of tnqe_apply_gate_noalloc (the
-library's gate + blocked Jacobi SVD + truncation on the GPU); the search is a
+library's gate, truncated block SVDs and truncation on the GPU); the search is a
 golden-section search (the paper names no optimiser) inside the best bracket
 of a coarse scan of [-pi/2, pi/2], plus the two endpoints, which are the
 FSWAP-like angles.
