@@ -256,7 +256,9 @@ int tnqe_graph_count(const tnqe_ctx* ctx);
  * H, S: M*M row-major, host; the upper triangle (i <= j) is used.
  * E: M doubles, the rank_kept ascending eigenvalues first, the rest NaN.
  * C: M*M row-major, column k = eigenvector k (C^T S C = I), zero beyond rank.
- * kappa1 = |c_1|^2 / sqrt(E_1^2 + 1) (App. A2).  Outputs are host memory. */
+ * kappa1 = |c_1|^2 / sqrt(E_1^2 + 1) (App. A2).  Outputs are host memory.
+ * A NaN or an infinity in the triangle used returns TNQE_ERR_NOCONV (outputs
+ * NaN, rank 0). */
 tnqe_status tnqe_solve(tnqe_ctx* ctx, const double* H, const double* S, int M,
                        double* E, double* C, int* rank_kept, double* kappa1);
 
