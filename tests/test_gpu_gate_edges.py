@@ -1,0 +1,87 @@
+"""The gate's truncation at the ends of its arguments' ranges (tnqe_apply_gate_noalloc with the identity gate on blocks
+of chosen size and spectrum), against NumPy's SVD or against the same call in the middle of the range."""
+import numpy as np
+import pytest
+
+from paper_2404_10223_gb300 import inputs, tnqe
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    import os
+    from paper_2404_10223_gb300 import build as B
+    if not os.path.exists(B.LIB):
+        B.build()
+    tnqe.load()
+
+
+def gate(A, B, q, side, chi_max, cutoff):
+    import torch
+    dA, dB = (torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in (A, B))
+    chl, chm, chr_ = A.shape[0], A.shape[2], B.shape[2]
+    Ao = torch.zeros(chl * 4 * chi_max, dtype=torch.float64, device="cuda")
+    Bo = torch.zeros(chi_max * 4 * chr_, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    k, _, disc = tnqe.tnqe_apply_gate_noalloc(dA.data_ptr(), dB.data_ptr(), chl, chm, chr_, *q, 1.0, 0.0, side,
+                                              chi_max, cutoff, 60, Ao.data_ptr(), Bo.data_ptr(), 0)
+    return (Ao[: chl * 4 * k].cpu().numpy().reshape(chl, 4, k), Bo[: k * 4 * chr_].cpu().numpy().reshape(k, 4, chr_),
+            k, disc)
+
+
+def blocks(shapes, spectra, rng):
+    """A two-site tensor with one block per (rows, cols), local states 3, 3, charges that do not couple."""
+    rows, cols, rs = ([0] + list(np.cumsum(x)) for x in
+                      ([s[0] for s in shapes], [s[1] for s in shapes], [len(x) for x in spectra]))
+    A, B = np.zeros((rows[-1], 4, rs[-1])), np.zeros((rs[-1], 4, cols[-1]))
+    q = [[], [], []]
+    for b, ((m, n), sg) in enumerate(zip(shapes, spectra)):
+        r = len(sg)
+        A[rows[b]:rows[b + 1], 3, rs[b]:rs[b + 1]] = np.linalg.qr(rng.normal(size=(m, r)))[0]
+        B[rs[b]:rs[b + 1], 3, cols[b]:cols[b + 1]] = np.asarray(sg)[:, None] * np.linalg.qr(rng.normal(size=(n, r)))[0].T
+        for x, (base, count) in enumerate([(17, m), (34, r), (51, n)]):
+            q[x] += [base + 3 * b] * count
+    return A, B, q
+
+
+@pytest.mark.parametrize("cutoff", [1.0, 1.5, 10.0, 1e300])
+@pytest.mark.parametrize("n", [4, 24, 90])
+@pytest.mark.parametrize("side", [0, 1])
+def test_a_cutoff_of_one_and_more_keeps_the_largest_singular_value(cutoff, n, side):
+    rng = np.random.default_rng(n)
+    A, B, q = blocks([(n + 3, n)], [1.0 - 0.9 * np.arange(n) / n], rng)
+    An, Bn, k, disc = gate(A, B, q, side, n, cutoff)
+    th = np.tensordot(A, B, axes=([2], [0]))[:, 3, 3, :]
+    u, sg, vt = np.linalg.svd(th)
+    assert k == 1
+    # FP64 rounding of either SVD over the gap at the cut (0.9 / n)
+    assert np.abs(np.tensordot(An, Bn, axes=([2], [0]))[:, 3, 3, :] - sg[0] * np.outer(u[:, 0], vt[0])).max() <= 1e-15 * n ** 2
+    assert abs(disc - (sg[1:] ** 2).sum()) <= 1e-12 * n
+
+
+@pytest.mark.parametrize("cutoff", [0.5, 1.0, 2.0])
+def test_a_cutoff_of_one_and_more_compares_narrow_and_wide_blocks(cutoff):
+    rng = np.random.default_rng(3)
+    A, B, q = blocks([(5, 4), (30, 24), (6, 4)], [[0.9, 0.3, 0.2, 0.1], np.linspace(1.0, 0.1, 24), [0.8, 0.1, 0.1, 0.05]], rng)
+    An, Bn, k, _ = gate(A, B, q, 0, 64, cutoff)
+    s = np.concatenate([[0.9, 0.3, 0.2, 0.1], np.linspace(1.0, 0.1, 24), [0.8, 0.1, 0.1, 0.05]])
+    kept = np.sort(np.linalg.norm(An.reshape(-1, k), axis=0))[::-1]
+    ref = np.sort(s)[::-1][: max(1, int((s > cutoff).sum()))]
+    assert k == len(ref) and np.abs(kept - ref).max() <= 1e-14
+
+
+@pytest.mark.parametrize("cutoff", [float("nan"), 1.5, 1e200])
+def test_rotations_with_such_a_cutoff_keep_one_column_a_bond(cutoff):
+    w = inputs.make_workload(6, 3, 3, 12, 2, [16, 16], seed=5)
+    ref = None
+    for ct in (1.0 - 1e-9, cutoff):                  # below 1 by less than any gap: the largest alone is above it
+        with tnqe.Context(w.h1, w.eri, w.N, w.n_alpha, w.n_beta, cutoff=ct) as g:
+            for m in w.mps:
+                g.add_mps(m.tensors, m.U)
+            g.rotate(0, 1)
+            got = g.get_rotated()
+        assert all(t.shape[2] == 1 for t in got)
+        if ref is not None:
+            assert all(np.array_equal(a, b) for a, b in zip(ref, got))
+        ref = got
