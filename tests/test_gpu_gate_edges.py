@@ -85,3 +85,21 @@ def test_rotations_with_such_a_cutoff_keep_one_column_a_bond(cutoff):
         if ref is not None:
             assert all(np.array_equal(a, b) for a, b in zip(ref, got))
         ref = got
+
+
+@pytest.mark.parametrize("e", [-900, -600, -450, 450, 600, 900, 1000])
+@pytest.mark.parametrize("n", [4, 24, 60, 90])
+@pytest.mark.parametrize("side", [0, 1])
+def test_a_tensor_times_a_power_of_two_gives_the_same_bits(e, n, side):
+    """The squares of the singular values leave the range of FP64 beyond 2^+-512; the singular values do not."""
+    rng = np.random.default_rng(n)
+    two = 2 if n <= 60 else 1                         # bonds of up to 128
+    A, B, q = blocks([(n + 3, n), (n, n + 2)][:two], [1.0 - 0.9 * np.arange(n) / n, 0.7 - 0.6 * np.arange(n) / n][:two], rng)
+    keep = n // 2 + 1
+    An, Bn, k, disc = gate(A, B, q, side, keep, 1e-14)
+    As, Bs, ks, ds = gate(np.ldexp(A, e), B, q, side, keep, 1e-14)
+    assert k == ks == keep
+    # the factor with the singular values takes the power of two
+    assert np.array_equal(np.ldexp(An, e if side == 0 else 0), As) and np.array_equal(np.ldexp(Bn, e if side == 1 else 0), Bs)
+    if abs(e) < 500:
+        assert ds == np.ldexp(disc, 2 * e)
