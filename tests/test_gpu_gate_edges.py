@@ -103,3 +103,25 @@ def test_a_tensor_times_a_power_of_two_gives_the_same_bits(e, n, side):
     assert np.array_equal(np.ldexp(An, e if side == 0 else 0), As) and np.array_equal(np.ldexp(Bn, e if side == 1 else 0), Bs)
     if abs(e) < 500:
         assert ds == np.ldexp(disc, 2 * e)
+
+
+@pytest.mark.parametrize("n", [2, 4, 5, 8, 9, 24, 60, 90])
+@pytest.mark.parametrize("close", [1e-3, 1e-6, 1e-9])
+@pytest.mark.parametrize("tall", [False, True])
+@pytest.mark.parametrize("side", [0, 1])
+def test_pairs_of_close_singular_values_leave_both_factors_orthogonal(n, close, tall, side):
+    """The isometric factor is V of the block for one orientation and W / sigma for the other."""
+    worst = 0.0
+    for seed in range(12 if n < 10 else 3):
+        rng = np.random.default_rng([n, seed])
+        sg = np.linspace(1.0, 0.2, n)
+        sg[1::2] = sg[0:2 * (n // 2):2] * (1.0 - close)
+        A, B, q = blocks([(n + 3, n) if tall else (n, n + 3)], [sg], rng)
+        An, Bn, k, _ = gate(A, B, q, side, n, 1e-14)
+        assert k == n
+        th = np.tensordot(A, B, axes=([2], [0]))
+        assert np.abs(np.tensordot(An, Bn, axes=([2], [0])) - th).max() <= 1e-15 * (n + 3)
+        X = Bn.reshape(k, -1) if side == 0 else An.reshape(-1, k).T
+        worst = max(worst, np.abs(X @ X.T - np.eye(k)).max())
+    # pairs are rotated down to m eps, and the last sweep leaves as much; W of wider blocks is a double-float product
+    assert worst <= 4.0 * (n + 3) * 2.0 ** -52 + (n > 8) * 4.0 * 2.0 ** -48
