@@ -22,7 +22,10 @@
 //      the update only need FP32).  It converges quadratically in the kept vectors and
 //      by 1e-6 over the relative distance of the eigenvalues along the dropped ones,
 //      whose eigenvalues stay FP32: on the gates of N = 14, chi = 128 states |t| is at
-//      most 1e-4, then 1e-8, so two corrections, sometimes three.  Last, the kept
+//      most 1e-4, then 1e-8, so two corrections, sometimes three.  x, w and lambda are
+//      FP64 (with double-floats of 48 bits the vectors and the truncated tensor were off
+//      by up to 1e-14, 9 to 24 columns by 1.5 times an FP64 Jacobi SVD; now by 1e-15 and
+//      a quarter of it, for 1.5 to 4 % of the time of a call).  Last, the kept
 //      vectors are orthonormalised by their inner products (I + (I - X^T X) / 2): the
 //      corrections alone leave 1e-13, and the matrix elements ten times the rounding
 //      error of an FP64 SVD.
@@ -35,15 +38,13 @@
 // an exact BF16 number, a digit product is at most 2^14 and the sums of one order are
 // integers below 2^24, so FP32 accumulation is exact, and seven digits (resolution
 // 2^-54 of the block's largest entry) with the 28 products of order up to 8 carry the
-// accuracy of double-float arithmetic (48 bits) or better.  A multiply-add costs 28/2048
+// accuracy of FP64 sums.  A multiply-add costs 28/2048
 // of a warp-wide mma against 12 FP32 instructions in double-float and 64 issue cycles
 // in FP64 (GB300's FP64 rate is 1/64 of its FP32 rate).  mma.sync and not tcgen05: the
 // blocks are 10 to 80 wide and eight to thirty columns are kept, far below a tcgen05
 // tile, and the operands of a warp come straight from L2 in fragment order.
 #pragma once
 #include <cuda_runtime.h>
-
-#include "df.cuh"
 
 namespace tnqe {
 namespace {
@@ -92,24 +93,6 @@ __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
   return o;
 }
 
-// s + e accumulates a b (double-floats): the compensated dot product of Ogita, Rump
-// and Oishi (SIAM J. Sci. Comput. 26 (2005) 1955), as accurate as twice FP32.
-__device__ __forceinline__ void dot2_step(float2 a, float2 b, float& s, float& e) {
-  const float p = __fmul_rn(a.x, b.x);
-  float pe = __fmaf_rn(a.x, b.x, -p);
-  float t, u;
-  dfa::two_sum(s, p, t, u);
-  s = t;
-  pe = __fmaf_rn(a.x, b.y, pe);
-  pe = __fmaf_rn(a.y, b.x, pe);
-  e = __fadd_rn(e, __fadd_rn(u, pe));
-}
-__device__ __forceinline__ float2 df_pair(float s, float e) {
-  float2 r;
-  dfa::two_sum(s, e, r.x, r.y);
-  return r;
-}
-
 // Uniform in [-1, 1] from a pair of indices (a start vector only has to be generic).
 __device__ __forceinline__ float eig_noise(unsigned i, unsigned u) {
   unsigned h = i * 0x9E3779B1u ^ (u + 0x7F4A7C15u) * 0x85EBCA77u;
@@ -124,22 +107,13 @@ __device__ __forceinline__ float eig_noise(unsigned i, unsigned u) {
 // ----------------------------------------------------------------------------- digits and mma fragments
 // A value v, |v| < 2, is the integer I = v 2^54 and I = sum_{s=1..7} d_s 2^(8 (7 - s)), d_s in
 // [-128, 128]: v = sum d_s 2^(2 - 8 s).
-__device__ __forceinline__ long long fix_float(float x, int ex) {   // x 2^(54 - ex), |x| < 2^(1 + ex)
-  const unsigned b = (unsigned)__float_as_int(x);
-  const int e = (int)((b >> 23) & 255);
-  const long long m = e ? (long long)((b & 0x7fffffu) | 0x800000u) : 0;
-  const int sh = e - 96 - ex;
-  const long long v = sh >= 0 ? m << min(sh, 40) : (sh > -25 ? m >> -sh : 0);
-  return (b >> 31) ? -v : v;
-}
-__device__ __forceinline__ long long fix_df(float2 v, int ex) { return fix_float(v.x, ex) + fix_float(v.y, ex); }
-// x / 2^ex 2^54 of a double, |x| < 2^(1 + ex)
+// x / 2^ex 2^54 of a double, |x| < 2^(1 + ex), to the nearest integer
 __device__ __forceinline__ long long fix_double(double x, int ex) {
   const long long b = __double_as_longlong(x);
   const int e = (int)((b >> 52) & 2047);
   const long long m = e ? ((b & 0xfffffffffffffll) | 0x10000000000000ll) : 0;
   const int sh = e - 1023 - ex + 2;
-  const long long v = sh >= 0 ? m << min(sh, 10) : (sh > -54 ? m >> -sh : 0);
+  const long long v = sh >= 0 ? m << min(sh, 10) : (sh > -54 ? (m + (1ll << (-sh - 1))) >> -sh : 0);
   return b < 0 ? -v : v;
 }
 // the digits of a pair of integers as BF16 pairs (first in the low half)
@@ -206,22 +180,22 @@ __device__ __noinline__ void eig_digits(const Team tm, const double* raw, int m,
   tm.sync();
 }
 
-// B-operand fragments of the columns k = 0..kp-1 of V (column k at k ldv, double-floats, |entries| <
+// B-operand fragments of the columns k = 0..kp-1 of V (column k at k ldv, |entries| <
 // 2^(1 + exs[k]), exs null: 2; length K padded with zeros to a multiple of 16): the 16 x 8 tile (kt, jt)
 // has its digits at ((kt JT + jt) ND + s) 32 + lane.
 template <int ND, class Team>
-__device__ __noinline__ void eig_digits_cols(const Team tm, const float2* V, int ldv, int K, int kp, const int* exs,
+__device__ __noinline__ void eig_digits_cols(const Team tm, const double* V, int ldv, int K, int kp, const int* exs,
                                              uint2* D) {
   const int lane = threadIdx.x & 31, warp = tm.rank() >> 5, nw = tm.size() >> 5;
   const int kt = pad16(K) >> 4, jt = kp >> 3, g = lane >> 2, t2 = 2 * (lane & 3);
   for (int t = warp; t < kt * jt; t += nw) {
     const int k = t / jt, j = t % jt;
     const int ex = exs ? exs[8 * j + g] : 0;
-    const float4* p = reinterpret_cast<const float4*>(V + (size_t)(8 * j + g) * ldv + 16 * k + t2);
-    const float4 lo = p[0], hi = p[4];
+    const double2* p = reinterpret_cast<const double2*>(V + (size_t)(8 * j + g) * ldv + 16 * k + t2);
+    const double2 lo = p[0], hi = p[4];
     unsigned a[EIG_DIG], b[EIG_DIG];
-    digits_pair(fix_df(make_float2(lo.x, lo.y), ex), fix_df(make_float2(lo.z, lo.w), ex), a);
-    digits_pair(fix_df(make_float2(hi.x, hi.y), ex), fix_df(make_float2(hi.z, hi.w), ex), b);
+    digits_pair(fix_double(lo.x, ex), fix_double(lo.y, ex), a);
+    digits_pair(fix_double(hi.x, ex), fix_double(hi.y, ex), b);
     uint2* d = D + (size_t)t * ND * 32 + lane;
 #pragma unroll
     for (int s = 0; s < ND; ++s) d[s * 32] = make_uint2(a[s], b[s]);
@@ -265,19 +239,23 @@ __device__ __forceinline__ void mma_tile(const uint4* A, const uint2* D, int it,
         if (i + s + 2 <= NS) mma_bf16(acc[i + s], a[i], b[s]);
   }
 }
-// The sums of all orders as a double-float, times 2^e (smallest order first).
+// 2^e, e in [-1022, 1023]
+__device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+// i as a double, |i| < 2^51 (one FP64 addition; the conversion instruction would be two)
+__device__ __forceinline__ double small_double(long long i) {
+  return __longlong_as_double(0x4338000000000000ll + i) - 6755399441055744.0;
+}
+// The sums of all orders, rounded once to FP64: the orders up to 4 and those above as two integers (at most 2^48).
 template <int NS>
-__device__ __forceinline__ float2 mma_value(const float (&acc)[NS - 1][4], int q, int e) {
-  float2 v = make_float2(0.f, 0.f);
+__device__ __forceinline__ double mma_value(const float (&acc)[NS - 1][4], int q) {
+  long long hi = 0, lo = 0;
 #pragma unroll
-  for (int o = NS - 2; o >= 0; --o) {
-    const float x = acc[o][q] * __int_as_float((127 + 4 - 8 * (o + 2)) << 23);
-    float s, r;
-    dfa::two_sum(x, v.x, s, r);
-    v = dfa::fast_two_sum(s, __fadd_rn(r, v.y));
+  for (int o = 0; o < NS - 1; ++o) {
+    const long long x = __float2int_rn(acc[o][q]);
+    if (o < 3) hi = (hi << 8) + x;
+    else lo = (lo << 8) + x;
   }
-  const float f = __int_as_float((127 + e) << 23);
-  return make_float2(v.x * f, v.y * f);
+  return fma(small_double(lo), pow2(4 - 8 * NS), small_double(hi) * pow2(-28));
 }
 
 // ----------------------------------------------------------------------------- Gram matrix
@@ -961,7 +939,7 @@ __device__ int eig_start(const Team& tm, const uint4* At, int m, int n, float* a
 // W (column k at k ldw, rows padded to 16) = B X from the digits of B (A) and of X (D): NA, NB, NS
 // as for mma_tile.
 template <int NA, int NB, int NS, class Team>
-__device__ __noinline__ void eig_bx(const Team tm, const uint4* A, const uint2* D, int m, int n, int kp, float2* W,
+__device__ __noinline__ void eig_bx(const Team tm, const uint4* A, const uint2* D, int m, int n, int kp, double* W,
                                     int ldw) {
   const int lane = threadIdx.x & 31, warp = tm.rank() >> 5, nw = tm.size() >> 5;
   const int mt = pad16(m) >> 4, KT = pad16(n) >> 4, JT = kp >> 3, g = lane >> 2, t2 = 2 * (lane & 3);
@@ -970,14 +948,14 @@ __device__ __noinline__ void eig_bx(const Team tm, const uint4* A, const uint2* 
     float acc[NS - 1][4];
     mma_tile<NA, NB, NS>(A, D, it, j, KT, JT, lane, acc);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) W[(8 * j + t2 + (q & 1)) * ldw + 16 * it + g + 8 * (q >> 1)] = mma_value<NS>(acc, q, 0);
+    for (int q = 0; q < 4; ++q) W[(8 * j + t2 + (q & 1)) * ldw + 16 * it + g + 8 * (q >> 1)] = mma_value<NS>(acc, q);
   }
   tm.sync();
 }
 // R (column k at k ld) = B^T W - X lambda from the digits of B^T (At) and of W (D, scaled by 2^-exs[k]).
 template <int NA, int NB, int NS, class Team>
 __device__ __noinline__ void eig_residual(const Team tm, const uint4* At, const uint2* D, int m, int n, int kp,
-                                          const float2* Xd, int ldx, const float2* lk, const int* exs, float* R,
+                                          const double* Xd, int ldx, const double* lk, const int* exs, float* R,
                                           int ld) {
   EIG_SHARED(lk);
   EIG_SHARED(R);
@@ -985,7 +963,7 @@ __device__ __noinline__ void eig_residual(const Team tm, const uint4* At, const 
   const int nt = pad16(n) >> 4, KT = pad16(m) >> 4, JT = kp >> 3, g = lane >> 2, t2 = 2 * (lane & 3);
   for (int t = warp; t < nt * JT; t += nw) {
     const int it = t % nt, j = t / nt;
-    float2 xv[4];
+    double xv[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) xv[q] = Xd[(8 * j + t2 + (q & 1)) * ldx + 16 * it + g + 8 * (q >> 1)];
     float acc[NS - 1][4];
@@ -993,43 +971,38 @@ __device__ __noinline__ void eig_residual(const Team tm, const uint4* At, const 
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int k = 8 * j + t2 + (q & 1), c = 16 * it + g + 8 * (q >> 1);
-      const float2 lx = dfa::mul(lk[k], xv[q]);
-      const float2 df = dfa::add(mma_value<NS>(acc, q, exs[k]), make_float2(-lx.x, -lx.y));
-      if (c < ld) R[k * ld + c] = c < n ? df.x + df.y : 0.f;
+      const float r = (float)fma(-lk[k], xv[q], mma_value<NS>(acc, q) * pow2(exs[k]));
+      if (c < ld) R[k * ld + c] = c < n ? r : 0.f;
     }
   }
   tm.sync();
 }
-// |column k|^2 of V (column k at k ldv, length K) as a double-float: eight lanes per column; f(k, value)
-// runs on one lane.
+// |column k|^2 of V (column k at k ldv, length K): eight lanes per column; f(k, value) runs on one lane.
 template <class Team, class F>
-__device__ __forceinline__ void eig_norms(const Team& tm, const float2* V, int ldv, int K, int kp, F f) {
+__device__ __forceinline__ void eig_norms(const Team& tm, const double* V, int ldv, int K, int kp, F f) {
   const int lane = threadIdx.x & 31, warp = tm.rank() >> 5, nw = tm.size() >> 5;
   for (int t = warp; t < kp / 4; t += nw) {
     const int k = 4 * t + (lane >> 3);
-    const float2* src = V + (size_t)k * ldv;
-    float s = 0.f, er = 0.f;
+    const double* src = V + (size_t)k * ldv;
+    double l = 0.0;
 #pragma unroll 4
-    for (int r = lane & 7; r < K; r += 8) {
-      const float2 v = src[r];
-      dot2_step(v, v, s, er);
-    }
-    float2 l = df_pair(s, er);
+    for (int r = lane & 7; r < K; r += 8) l = fma(src[r], src[r], l);
 #pragma unroll
-    for (int o = 4; o > 0; o >>= 1)
-      l = dfa::add(l, make_float2(__shfl_xor_sync(0xffffffffu, l.x, o), __shfl_xor_sync(0xffffffffu, l.y, o)));
+    for (int o = 4; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
     if ((lane & 7) == 0) f(k, l);
   }
 }
 // T (row i at i kp) = X R / (lambda_k - lambda_i), half the norm's defect ek on the diagonal: lanes are
-// vectors i.  lam: the eigenvalues of the discarded vectors, FP32 (1e-6 lam[0] or better): a correction leaves
-// 1e-6 lam[0] / |lambda_k - lambda_i| of itself along those.  Returns the largest |entry|, along
+// vectors i.  lk: the eigenvalues of the kept vectors, lh the same in FP32; lam: those of the discarded vectors, FP32
+// (1e-6 lam[0] or better): a correction leaves 1e-6 lam[0] / |lambda_k - lambda_i| of itself along those.  Returns the largest |entry|, along
 // discarded vectors closer than 1e-3 lam[0] times 1e-3 lam[0] / |lambda_k - lambda_i|.
 template <class Team>
 __device__ __noinline__ float eig_angles(const Team tm, const float* X, const float* R, int n, int ld, int kc, int kp,
-                                         const float2* lk, const float* ek, const float* lam, float* T) {
+                                         const double* lk, const float* lh, const float* ek, const float* lam,
+                                         float* T) {
   EIG_SHARED(R);
   EIG_SHARED(lk);
+  EIG_SHARED(lh);
   EIG_SHARED(ek);
   EIG_SHARED(lam);
   EIG_SHARED(T);
@@ -1057,7 +1030,7 @@ __device__ __noinline__ float eig_angles(const Team tm, const float* X, const fl
 #pragma unroll
     for (int q = 0; q < EIG_TC; ++q) s[q] = s2[q].x + s2[q].y;
     if (i < n) {
-      const float2 li = i < kc ? lk[i] : make_float2(lam[i], 0.f);
+      const double li = i < kc ? lk[i] : 0.0;
       const float near = i < kc ? 0.f : 1e-3f * lam[0];
       float o[EIG_TC];
 #pragma unroll
@@ -1068,7 +1041,7 @@ __device__ __noinline__ float eig_angles(const Team tm, const float* X, const fl
           if (i == k) {
             v = 0.5f * ek[k];
           } else {
-            const float den = (lk[k].x - li.x) + (lk[k].y - li.y);
+            const float den = i < kc ? (float)(lk[k] - li) : lh[k] - lam[i];
             v = den != 0.f ? __fdividef(s[q], den) : (s[q] == 0.f ? 0.f : 1e30f);
             if (fabsf(den) < near) w = __fdividef(near, fabsf(den));
           }
@@ -1087,7 +1060,7 @@ __device__ __noinline__ float eig_angles(const Team tm, const float* X, const fl
 // T (row i at i kp, kc rows) = half the defect of the kept vectors' inner products, (I - X^T X) / 2: eight
 // lanes per pair.
 template <class Team>
-__device__ __noinline__ void eig_orth(const Team tm, const float2* Xd, int ldx, int n, int kc, int kp, float* T) {
+__device__ __noinline__ void eig_orth(const Team tm, const double* Xd, int ldx, int n, int kc, int kp, float* T) {
   EIG_SHARED(T);
   const int gl = tm.rank() & 7, ng = tm.size() >> 3, np = kc * (kc + 1) / 2;
   for (int x = tm.rank(); x < kc * kp; x += tm.size()) T[x] = 0.f;   // (columns beyond kc)
@@ -1099,17 +1072,15 @@ __device__ __noinline__ void eig_orth(const Team tm, const float2* Xd, int ldx, 
     while (k * (k + 1) / 2 > p) --k;
     while ((k + 2) * (k + 1) / 2 <= p) ++k;
     const int i = p - k * (k + 1) / 2;
-    const float2* a = Xd + (size_t)i * ldx;
-    const float2* b = Xd + (size_t)k * ldx;
-    float s = 0.f, er = 0.f;
+    const double* a = Xd + (size_t)i * ldx;
+    const double* b = Xd + (size_t)k * ldx;
+    double l = 0.0;
 #pragma unroll 2
-    for (int r = gl; r < n; r += 8) dot2_step(a[r], b[r], s, er);
-    float2 l = df_pair(s, er);
+    for (int r = gl; r < n; r += 8) l = fma(a[r], b[r], l);
 #pragma unroll
-    for (int o = 4; o > 0; o >>= 1)
-      l = dfa::add(l, make_float2(__shfl_xor_sync(0xffffffffu, l.x, o), __shfl_xor_sync(0xffffffffu, l.y, o)));
+    for (int o = 4; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
     if (gl == 0) {
-      const float e = 0.5f * __fadd_rn(__fadd_rn(i == k ? 1.f : 0.f, -l.x), -l.y);
+      const float e = 0.5f * (float)((i == k ? 1.0 : 0.0) - l);
       T[i * kp + k] = e;
       T[k * kp + i] = e;
     }
@@ -1119,14 +1090,14 @@ __device__ __noinline__ void eig_orth(const Team tm, const float2* Xd, int ldx, 
 // Xd (column k at k ldx) += X^T T (nv rows), and the FP32 vectors Xg (row k at k ld) follow: lanes are components.
 template <class Team>
 __device__ __noinline__ void eig_update(const Team tm, const float* X, const float* T, int nv, int n, int ld, int kc,
-                                        int kp, float2* Xd, int ldx, float* Xg) {
+                                        int kp, double* Xd, int ldx, float* Xg) {
   EIG_SHARED(T);
   const int lane = threadIdx.x & 31, warp = tm.rank() >> 5, nw = tm.size() >> 5;
   const int rc = (n + 31) >> 5, kcn = kp / EIG_TC;
   for (int t = warp; t < rc * kcn; t += nw) {
     const int i = (t % rc) * 32 + lane, k0 = (t / rc) * EIG_TC, ic = min(i, n - 1);
     float2 s2[EIG_TC / 2];
-    float2 xv[EIG_TC];
+    double xv[EIG_TC];
 #pragma unroll
     for (int q = 0; q < EIG_TC; ++q) xv[q] = Xd[(size_t)(k0 + q) * ldx + ic];
 #pragma unroll
@@ -1147,9 +1118,9 @@ __device__ __noinline__ void eig_update(const Team tm, const float* X, const flo
     if (i < n) {
 #pragma unroll
       for (int q = 0; q < EIG_TC; ++q) {
-        const float2 v = dfa::add(xv[q], make_float2(s[q], 0.f));
+        const double v = xv[q] + (double)s[q];
         Xd[(size_t)(k0 + q) * ldx + i] = v;
-        if (k0 + q < kc) Xg[(k0 + q) * ld + i] = v.x;
+        if (k0 + q < kc) Xg[(k0 + q) * ld + i] = (float)v;
       }
     }
   }
@@ -1159,21 +1130,22 @@ __device__ __noinline__ void eig_update(const Team tm, const float* X, const flo
 // Refines the first kc vectors of Xg (n x ld, one per row; updated) as described at the top.  A, At: the
 // digits of B and B^T; lam0 the approximate eigenvalues.  Outputs: Wout (column j at j m), Qout
 // (column j at j n) in FP64, the singular values in sig[0..kc).  Wd, Xd (kp columns of length m
-// and n padded to 16, double-floats), Dg (digits of either) and Xalt (n x ld floats) are global
+// and n padded to 16), Dg (digits of either) and Xalt (n x ld floats) are global
 // scratch, used where the arena is too small.  Returns 0, or 1 if the
 // corrections do not converge or the block does not fit.
 template <class Team>
 __device__ int eig_refine(const Team& tm, const uint4* A, const uint4* At, int m, int n, int kc, float* Xg,
-                          const float* lam0, float* arena, int words, float2* Wd, float2* Xd, uint2* Dg, float* Xalt,
+                          const float* lam0, float* arena, int words, double* Wd, double* Xd, uint2* Dg, float* Xalt,
                           double* Wout, double* Qout, double* sig, double scale) {
   const int tr = tm.rank(), ts = tm.size();
   const int ld = eig_ld(n), kp = eig_kp(kc), m16 = pad16(m), n16 = pad16(n);
-  // arena: lk (kp float2), ek and exs (kp), lam (ld), R (kp x ld), then the digits or, after them, T
+  // arena: lk (kp doubles), lh, ek and exs (kp), lam (ld), R (kp x ld), then the digits or, after them, T
   // (n x kp) and X (n x ld)
-  const int fix = 4 * kp + ld + kp * ld, dig = m16 * kp * EIG_DIG / 2, tx = n * kp;
+  const int fix = 5 * kp + ld + kp * ld, dig = m16 * kp * EIG_DIG / 2, tx = n * kp;
   if (fix + tx > words) return 1;
-  float2* lk = reinterpret_cast<float2*>(arena);
-  float* ek = arena + 2 * kp;
+  double* lk = reinterpret_cast<double*>(arena);
+  float* lh = arena + 2 * kp;
+  float* ek = lh + kp;
   int* exs = reinterpret_cast<int*>(ek + kp);
   float* lam = ek + 2 * kp;
   float* R = lam + ld;
@@ -1184,16 +1156,16 @@ __device__ int eig_refine(const Team& tm, const uint4* A, const uint4* At, int m
   // what is left behind the larger of the two takes the columns themselves
   int at = fix + max(fix + dig <= words ? dig : 0, tx + (xin ? n * ld : 0));
   if (at + 2 * n16 * kp <= words) {
-    Xd = reinterpret_cast<float2*>(arena + at);
+    Xd = reinterpret_cast<double*>(arena + at);
     at += 2 * n16 * kp;
   }
-  if (at + 2 * m16 * kp <= words) Wd = reinterpret_cast<float2*>(arena + at);
+  if (at + 2 * m16 * kp <= words) Wd = reinterpret_cast<double*>(arena + at);
   for (int x = tr; x < n16 * kp; x += ts) {
     const int k = x / n16, c = x % n16;
     float v = (k < kc && c < n) ? Xg[k * ld + c] : 0.f;
     // four digits carry the start vectors: entries below 2^-7 are rounded to 2^-30
     if (fabsf(v) < 0.0078125f) v = __fsub_rn(__fadd_rn(v, 0.01171875f), 0.01171875f);
-    Xd[x] = make_float2(v, 0.f);
+    Xd[x] = (double)v;
   }
   for (int x = tr; x < n; x += ts) lam[x] = lam0[x];
   tm.sync();
@@ -1206,11 +1178,12 @@ __device__ int eig_refine(const Team& tm, const uint4* A, const uint4* At, int m
       eig_digits_cols<EIG_DIG>(tm, Xd, n16, n, kp, nullptr, D);
       eig_bx<EIG_DIG, EIG_DIG, EIG_DIG + 1>(tm, A, D, m, n, kp, Wd, m16);
     }
-    eig_norms(tm, Wd, m16, m, kp, [&](int k, float2 l) {
+    eig_norms(tm, Wd, m16, m, kp, [&](int k, double l) {
       lk[k] = l;
-      exs[k] = (((__float_as_int(l.x) >> 23) & 255) - 127) >> 1;     // |w| < 2^(1 + exs)
+      lh[k] = (float)l;
+      exs[k] = (((__double2hiint(l) >> 20) & 2047) - 1023) >> 1;     // |w| < 2^(1 + exs)
     });
-    eig_norms(tm, Xd, n16, n, kp, [&](int k, float2 l) { ek[k] = __fadd_rn(__fadd_rn(1.f, -l.x), -l.y); });
+    eig_norms(tm, Xd, n16, n, kp, [&](int k, double l) { ek[k] = (float)(1.0 - l); });
     tm.sync();
     if (it == 0) {
       eig_digits_cols<6>(tm, Wd, m16, m, kp, exs, D);
@@ -1220,7 +1193,7 @@ __device__ int eig_refine(const Team& tm, const uint4* A, const uint4* At, int m
       eig_residual<EIG_DIG, EIG_DIG, EIG_DIG + 1>(tm, At, D, m, n, kp, Xd, n16, lk, exs, R, ld);
     }
     eig_copy(tm, Xg, n * ld, X);
-    const float worst = eig_angles(tm, X, R, n, ld, kc, kp, lk, ek, lam, T);
+    const float worst = eig_angles(tm, X, R, n, ld, kc, kp, lk, lh, ek, lam, T);
     if (!(worst < 0.25f)) return 1;
     eig_update(tm, X, T, n, n, ld, kc, kp, Xd, n16, Xg);
     if (worst <= EIG_ACCEPT) break;
@@ -1233,11 +1206,11 @@ __device__ int eig_refine(const Team& tm, const uint4* A, const uint4* At, int m
   eig_update(tm, X, T, kc, n, ld, kc, kp, Xd, n16, Xg);
   eig_digits_cols<EIG_DIG>(tm, Xd, n16, n, kp, nullptr, D);
   eig_bx<EIG_DIG, EIG_DIG, EIG_DIG + 1>(tm, A, D, m, n, kp, Wd, m16);
-  eig_norms(tm, Wd, m16, m, kp, [&](int k, float2 l) {
-    if (k < kc) sig[k] = sqrt(dfa::to_double(l)) * scale;
+  eig_norms(tm, Wd, m16, m, kp, [&](int k, double l) {
+    if (k < kc) sig[k] = sqrt(l) * scale;
   });
-  for (int x = tr; x < m * kc; x += ts) Wout[x] = dfa::to_double(Wd[(size_t)(x / m) * m16 + x % m]);
-  for (int x = tr; x < n * kc; x += ts) Qout[x] = dfa::to_double(Xd[(size_t)(x / n) * n16 + x % n]);
+  for (int x = tr; x < m * kc; x += ts) Wout[x] = Wd[(size_t)(x / m) * m16 + x % m];
+  for (int x = tr; x < n * kc; x += ts) Qout[x] = Xd[(size_t)(x / n) * n16 + x % n];
   tm.sync();
   return 0;
 }

@@ -125,3 +125,23 @@ def test_pairs_of_close_singular_values_leave_both_factors_orthogonal(n, close, 
         worst = max(worst, np.abs(X @ X.T - np.eye(k)).max())
     # pairs are rotated down to m eps, and the last sweep leaves as much; W of wider blocks is a double-float product
     assert worst <= 4.0 * (n + 3) * 2.0 ** -52 + (n > 8) * 4.0 * 2.0 ** -48
+
+
+@pytest.mark.parametrize("n", [9, 12, 24, 40, 60, 90])
+@pytest.mark.parametrize("tall", [False, True])
+@pytest.mark.parametrize("side", [0, 1])
+def test_truncated_factors_are_orthonormal_to_fp64(n, tall, side):
+    """Well separated singular values, a third of them kept: what is rounded is FP64 vectors of unit length (an error of
+    2^-53 of each entry, sums of n terms in random order)."""
+    rng = np.random.default_rng(n)
+    sg = 1.0 - 0.9 * np.arange(n) / n
+    A, B, q = blocks([(n + 3, n) if tall else (n, n + 3)], [sg], rng)
+    An, Bn, k, disc = gate(A, B, q, side, n // 3, 1e-14)
+    X = (Bn.reshape(k, -1) if side == 0 else An.reshape(-1, k).T).astype(np.longdouble)
+    W = (An.reshape(-1, k).T if side == 0 else Bn.reshape(k, -1)).astype(np.longdouble)
+    assert np.abs(X @ X.T - np.eye(k)).max() <= 2.0 ** -52 * np.sqrt(n)
+    G = W @ W.T
+    d = np.sqrt(np.diag(G))
+    assert np.abs(d - sg[:k]).max() <= 2.0 ** -52 * np.sqrt(n)     # the tensor itself is rounded as much
+    # the inner products of W are those of X times the squares of the singular values (at most 1, at least 0.46)
+    assert np.abs(G / np.outer(d, d) - np.eye(k)).max() <= 2.0 ** -51 * np.sqrt(n)
