@@ -68,6 +68,12 @@ __device__ __forceinline__ float warp_max_f(float v) {
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
 }
+// The larger of two values, a NaN if either is one.
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
 // Row stride of the n x n FP32 arrays: a multiple of 4 (16-byte rows) and 4 mod 8, so
 // that 16-byte accesses of eight consecutive rows fall into distinct banks.
 __host__ __device__ __forceinline__ int eig_ld(int n) {
@@ -826,14 +832,13 @@ __device__ __noinline__ float eig_defect(const Team tm, const float* X, int n, i
         const int i = 4 * iq + a, j = 4 * jq + b;
         if (i < n && j < n && i <= j) {
           const float v = (i == j ? 1.f : 0.f) - (acc[a][b].x + acc[a][b].y);
-          worst = (fabsf(v) <= worst) ? worst : fabsf(v);      // NaN stays
+          worst = max_nan(worst, fabsf(v));
           E[i * ld + j] = v;
           E[j * ld + i] = v;
         }
       }
   }
-  if (!(worst >= 0.f)) worst = 1e30f;
-  worst = fminf(worst, 1e30f);
+  if (!(worst <= 1e30f)) worst = 1e30f;            // a NaN too
   return tm.max(worst);                            // ends with a team barrier
 }
 // out (row stride lo = ld) = X + E X / 2 over the vectors
@@ -1045,8 +1050,7 @@ __device__ __noinline__ float eig_angles(const Team tm, const float* X, const fl
             v = den != 0.f ? __fdividef(s[q], den) : (s[q] == 0.f ? 0.f : 1e30f);
             if (fabsf(den) < near) w = __fdividef(near, fabsf(den));
           }
-          w *= fabsf(v);
-          worst = (w <= worst) ? worst : w;
+          worst = max_nan(worst, w * fabsf(v));
         }
         o[q] = v;
       }
@@ -1054,8 +1058,8 @@ __device__ __noinline__ float eig_angles(const Team tm, const float* X, const fl
       *reinterpret_cast<float4*>(T + i * kp + k0 + 4) = make_float4(o[4], o[5], o[6], o[7]);
     }
   }
-  if (!(worst >= 0.f)) worst = 1e30f;
-  return tm.max(fminf(worst, 1e30f));
+  if (!(worst <= 1e30f)) worst = 1e30f;            // a NaN too
+  return tm.max(worst);
 }
 // T (row i at i kp, kc rows) = half the defect of the kept vectors' inner products, (I - X^T X) / 2: eight
 // lanes per pair.
