@@ -437,8 +437,9 @@ PairPlan* get_plan(tnqe_ctx* c, int i, int j) {
 
 int chi_rot_of(tnqe_ctx* c, int j) { return c->opt.chi_rot > 0 ? c->opt.chi_rot : c->mps[j]->chi; }
 
-// Launch the rotation of every (i, j), i != j, of `pairs`; results stay in rot_work.
-void run_rotations(tnqe_ctx* c, const std::vector<std::pair<int, int>>& pairs, RotBatch& rb, int pad_out) {
+// Launch the rotation of every (i, j), i != j, of `pairs`; results stay in rot_work.  weights: the discarded weights
+// are computed too.
+void run_rotations(tnqe_ctx* c, const std::vector<std::pair<int, int>>& pairs, RotBatch& rb, int pad_out, bool weights) {
   const int N = c->N;
   rb = RotBatch{};
   for (size_t p = 0; p < pairs.size(); ++p)
@@ -565,7 +566,7 @@ void run_rotations(tnqe_ctx* c, const std::vector<std::pair<int, int>>& pairs, R
     d.carve_cap = 0;
     d.meta = c->rot_meta.as<int>() + META_INTS * cluster * k;
     d.meta_cap = META_INTS;
-    d.discarded = ddisc;
+    d.discarded = weights ? ddisc : nullptr;
     d.status = dstat;
     d.flops = dflops;
     rb.work.push_back(d.work);
@@ -1654,7 +1655,7 @@ void enqueue_matrix_elements(tnqe_ctx* c, const std::vector<std::pair<int, int>>
   double* mS = split ? oS + di.size() : dS;
   record_event(c, c->ev[0]);
   RotBatch rb;
-  run_rotations(c, pm, rb, 1);
+  run_rotations(c, pm, rb, 1, false);
   for (const auto& p : pl) start_mpo(c, *c->mps[p.first]);   // builds not yet started run beside the rotation
   record_event(c, c->ev[1]);
   // The bra states' MPOs: their host builds started just above; the host
@@ -2491,7 +2492,7 @@ tnqe_status tnqe_rotate(tnqe_ctx* c, int i, int j, double* discarded_weight) {
       return TNQE_OK;
     }
     RotBatch rb;
-    run_rotations(c, {{i, j}}, rb, 0);
+    run_rotations(c, {{i, j}}, rb, 0, true);
     std::vector<std::vector<int>> dims;
     std::vector<double> disc;
     int st = 0;

@@ -94,7 +94,7 @@ struct RotDesc {
   long long carve_cap;
   int* meta;                      // scratch ints, meta_cap for each CTA of the pair
   long long meta_cap;
-  double* discarded;
+  double* discarded;              // NULL: the discarded weight is not wanted
   int* status;
   double* flops;                  // algorithmic FLOPs of this rotation (written at exit)
 };

@@ -156,7 +156,7 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint4& a, const ui
 // A-operand fragments of B (rows of B) in A and of B^T in At, tile by tile: the 16 x 16 tile
 // (it, kt) of a matrix with KT column tiles has its EIG_DIG digits at ((it KT + kt) EIG_DIG + s) 32
 // + lane.  raw: B column-major (m x n), |entries| < 2^(1 + ex).  A warp takes a tile of
-// B; its transpose comes from the registers (movmatrix).
+// B; its transpose comes from the registers (movmatrix) unless At is null.
 template <class Team>
 __device__ __noinline__ void eig_digits(const Team tm, const double* raw, int m, int n, int ex, uint4* A, uint4* At) {
   const int lane = threadIdx.x & 31, warp = tm.rank() >> 5, nw = tm.size() >> 5;
@@ -180,7 +180,7 @@ __device__ __noinline__ void eig_digits(const Team tm, const double* raw, int m,
 #pragma unroll
     for (int s = 0; s < EIG_DIG; ++s) {
       a[s * 32] = make_uint4(w[0][s], w[1][s], w[2][s], w[3][s]);
-      b[s * 32] = make_uint4(transpose8x8(w[0][s]), transpose8x8(w[2][s]), transpose8x8(w[1][s]), transpose8x8(w[3][s]));
+      if (At) b[s * 32] = make_uint4(transpose8x8(w[0][s]), transpose8x8(w[2][s]), transpose8x8(w[1][s]), transpose8x8(w[3][s]));
     }
   }
   tm.sync();
@@ -251,9 +251,10 @@ __device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + 
 __device__ __forceinline__ double small_double(long long i) {
   return __longlong_as_double(0x4338000000000000ll + i) - 6755399441055744.0;
 }
-// The sums of all orders, rounded once to FP64: the orders up to 4 and those above as two integers (at most 2^48).
+// The sums of all orders times 2^e, rounded once to FP64: the orders up to 4 and those above as two integers (at
+// most 2^48).
 template <int NS>
-__device__ __forceinline__ double mma_value(const float (&acc)[NS - 1][4], int q) {
+__device__ __forceinline__ double mma_value(const float (&acc)[NS - 1][4], int q, int e) {
   long long hi = 0, lo = 0;
 #pragma unroll
   for (int o = 0; o < NS - 1; ++o) {
@@ -261,7 +262,7 @@ __device__ __forceinline__ double mma_value(const float (&acc)[NS - 1][4], int q
     if (o < 3) hi = (hi << 8) + x;
     else lo = (lo << 8) + x;
   }
-  return fma(small_double(lo), pow2(4 - 8 * NS), small_double(hi) * pow2(-28));
+  return fma(small_double(lo), pow2(e + 4 - 8 * NS), small_double(hi) * pow2(e - 28));
 }
 
 // ----------------------------------------------------------------------------- Gram matrix
@@ -891,7 +892,7 @@ __device__ __forceinline__ void eig_copy(const Team& tm, const float* from, int 
 
 template <bool XS, class Team>
 __device__ int eig_start_at(const Team tm, const uint4* At, int m, int n, float* A, float* X, float* V, float* Xg,
-                            float* lamg, float2* Sg) {
+                            float* lamg, float2* Sg, float* trace) {
   const int tr = tm.rank(), ts = tm.size();
   const int ld = eig_ld(n);
   float* W = V + 2 * ld;
@@ -902,6 +903,12 @@ __device__ int eig_start_at(const Team tm, const uint4* At, int m, int n, float*
   float* lam = tau + ld;
   float* inorm = lam + ld;
   eig_gram(tm, At, m, n, A, ld);
+  if (tr < 32) {                                   // (this warp takes part in the first barrier of the reduction)
+    float t = 0.f;
+    for (int i = tr; i < n; i += 32) t += A[i * ld + i];
+    t = warp_sum_f(t);
+    if (tr == 0) *trace = t;
+  }
   eig_tridiag(tm, A, n, ld, V, W, P, d, e, tau, inorm + ld);
   const float sc = eig_values(tm, d, e, n, ld, reinterpret_cast<float2*>(P), lam);
   for (int x = tr; x < n * (ld - n); x += ts) X[(x / (ld - n)) * ld + n + x % (ld - n)] = 0.f;
@@ -928,16 +935,16 @@ __device__ int eig_start_at(const Team tm, const uint4* At, int m, int n, float*
 // `words` floats of shared memory (16-byte aligned); Xg (n x ld floats, one vector per
 // row, pad components zero, eigenvalues descending) and lamg (n floats) receive the result, Sg (n x
 // n pairs) and Xalt (n x ld floats, for X where the arena only holds A) are scratch, all
-// in global memory.  Returns 0, 1 if the block does not fit (no result), or 3 if X is not
+// in global memory; *trace gets the sum of all eigenvalues.  Returns 0, 1 if the block does not fit (no result), or 3 if X is not
 // orthonormal in the end (the eigenvalues hold).
 template <class Team>
 __device__ int eig_start(const Team& tm, const uint4* At, int m, int n, float* arena, int words, float* Xg, float* lamg,
-                         float2* Sg, float* Xalt) {
+                         float2* Sg, float* Xalt, float* trace) {
   const int ld = eig_ld(n);
   if (n > EIG_MAXN || n * ld + eig_vec_floats(n) > words) return 1;
   if (2 * n * ld + eig_vec_floats(n) <= words)
-    return eig_start_at<true>(tm, At, m, n, arena, arena + n * ld, arena + 2 * n * ld, Xg, lamg, Sg);
-  return eig_start_at<false>(tm, At, m, n, arena, Xalt, arena + n * ld, Xg, lamg, Sg);
+    return eig_start_at<true>(tm, At, m, n, arena, arena + n * ld, arena + 2 * n * ld, Xg, lamg, Sg, trace);
+  return eig_start_at<false>(tm, At, m, n, arena, Xalt, arena + n * ld, Xg, lamg, Sg, trace);
 }
 
 // ----------------------------------------------------------------------------- refinement
@@ -953,7 +960,7 @@ __device__ __noinline__ void eig_bx(const Team tm, const uint4* A, const uint2* 
     float acc[NS - 1][4];
     mma_tile<NA, NB, NS>(A, D, it, j, KT, JT, lane, acc);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) W[(8 * j + t2 + (q & 1)) * ldw + 16 * it + g + 8 * (q >> 1)] = mma_value<NS>(acc, q);
+    for (int q = 0; q < 4; ++q) W[(8 * j + t2 + (q & 1)) * ldw + 16 * it + g + 8 * (q >> 1)] = mma_value<NS>(acc, q, 0);
   }
   tm.sync();
 }
@@ -976,7 +983,7 @@ __device__ __noinline__ void eig_residual(const Team tm, const uint4* At, const 
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int k = 8 * j + t2 + (q & 1), c = 16 * it + g + 8 * (q >> 1);
-      const float r = (float)fma(-lk[k], xv[q], mma_value<NS>(acc, q) * pow2(exs[k]));
+      const float r = (float)fma(-lk[k], xv[q], mma_value<NS>(acc, q, exs[k]));
       if (c < ld) R[k * ld + c] = c < n ? r : 0.f;
     }
   }
@@ -1131,16 +1138,69 @@ __device__ __noinline__ void eig_update(const Team tm, const float* X, const flo
   tm.sync();
 }
 
+// |B - W X^T|^2 for the kc columns of W = B X, of which Wf has the digits over 2^ex as fragments of W and Xf those of X
+// (eig_digits): what the other singular values weigh, without the cancellation of a difference of norms (down to
+// 1e-4 of the block's: 2e-11 of the weight with double-float vectors, 1e-12 in FP64).  B = raw / 2^e with
+// inv = 2^-e, column-major.  tsum: 2 pad16(m) pad16(n) / 256 doubles of the team's memory.  The same on every
+// thread, and the same sum whatever the team's size.
+template <class Team>
+__device__ __noinline__ double eig_rest(const Team tm, const uint4* Wf, const uint4* Xf, int ex, const double* raw,
+                                        double inv, int m, int n, int kc, double* tsum) {
+  const int lane = threadIdx.x & 31, warp = tm.rank() >> 5, nw = tm.size() >> 5;
+  const int mt = pad16(m) >> 4, jt = (n + 7) >> 3, KT = pad16(kc) >> 4, g = lane >> 2, t2 = 2 * (lane & 3);
+  for (int t = warp; t < mt * jt; t += nw) {
+    const int it = t % mt, j8 = t / mt;
+    float acc[EIG_DIG][4];
+#pragma unroll
+    for (int o = 0; o < EIG_DIG; ++o)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[o][q] = 0.f;
+    for (int k = 0; k < KT; ++k) {
+      const uint4* ap = Wf + (size_t)(it * KT + k) * EIG_DIG * 32 + lane;
+      const uint4* bp = Xf + (size_t)((j8 >> 1) * KT + k) * EIG_DIG * 32 + lane;
+      uint4 a[EIG_DIG];
+      uint2 b[EIG_DIG];
+#pragma unroll
+      for (int s = 0; s < EIG_DIG; ++s) {
+        a[s] = ap[s * 32];
+        const uint4 v = bp[s * 32];
+        b[s] = (j8 & 1) ? make_uint2(v.y, v.w) : make_uint2(v.x, v.z);
+      }
+#pragma unroll
+      for (int i = 0; i < EIG_DIG; ++i)
+#pragma unroll
+        for (int s = 0; s < EIG_DIG; ++s)
+          if (i + s < EIG_DIG) mma_bf16(acc[i + s], a[i], b[s]);
+    }
+    double sum = 0.0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int r = 16 * it + g + 8 * (q >> 1), c = 8 * j8 + t2 + (q & 1);
+      const double d = r < m && c < n ? fma(raw[(size_t)c * m + r], inv, -mma_value<EIG_DIG + 1>(acc, q, ex)) : 0.0;
+      sum = fma(d, d, sum);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) tsum[t] = sum;
+  }
+  tm.sync();
+  double sum = 0.0;
+  for (int t = lane; t < mt * jt; t += 32) sum += tsum[t];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  return sum;
+}
+
 // Refines the first kc vectors of Xg (n x ld, one per row; updated) as described at the top.  A, At: the
 // digits of B and B^T; lam0 the approximate eigenvalues.  Outputs: Wout (column j at j m), Qout
 // (column j at j n) in FP64, the singular values in sig[0..kc).  Wd, Xd (kp columns of length m
 // and n padded to 16), Dg (digits of either) and Xalt (n x ld floats) are global
-// scratch, used where the arena is too small.  Returns 0, or 1 if the
-// corrections do not converge or the block does not fit.
+// scratch, used where the arena is too small.  *rest (if wanted) gets eig_rest of the block raw / scale (A and At are
+// overwritten for it).  Returns 0, or 1 if the corrections do not converge or the block does not fit.
 template <class Team>
-__device__ int eig_refine(const Team& tm, const uint4* A, const uint4* At, int m, int n, int kc, float* Xg,
+__device__ int eig_refine(const Team& tm, uint4* A, uint4* At, int m, int n, int kc, float* Xg,
                           const float* lam0, float* arena, int words, double* Wd, double* Xd, uint2* Dg, float* Xalt,
-                          double* Wout, double* Qout, double* sig, double scale) {
+                          double* Wout, double* Qout, double* sig, double scale, const double* raw, double* rest) {
   const int tr = tm.rank(), ts = tm.size();
   const int ld = eig_ld(n), kp = eig_kp(kc), m16 = pad16(m), n16 = pad16(n);
   // arena: lk (kp doubles), lh, ek and exs (kp), lam (ld), R (kp x ld), then the digits or, after them, T
@@ -1185,7 +1245,7 @@ __device__ int eig_refine(const Team& tm, const uint4* A, const uint4* At, int m
     eig_norms(tm, Wd, m16, m, kp, [&](int k, double l) {
       lk[k] = l;
       lh[k] = (float)l;
-      exs[k] = (((__double2hiint(l) >> 20) & 2047) - 1023) >> 1;     // |w| < 2^(1 + exs)
+      exs[k] = (((__double2hiint(l) >> 20) & 2047) - 1023) >> 1;     // |w| < 2^(1 + exs); a padding column -512
     });
     eig_norms(tm, Xd, n16, n, kp, [&](int k, double l) { ek[k] = (float)(1.0 - l); });
     tm.sync();
@@ -1215,6 +1275,16 @@ __device__ int eig_refine(const Team& tm, const uint4* A, const uint4* At, int m
   });
   for (int x = tr; x < m * kc; x += ts) Wout[x] = Wd[(size_t)(x / m) * m16 + x % m];
   for (int x = tr; x < n * kc; x += ts) Qout[x] = Xd[(size_t)(x / n) * n16 + x % n];
+  if (!rest || kc == n) {
+    tm.sync();
+    return 0;
+  }
+  int ex = exs[0];
+  for (int k = 1; k < kc; ++k) ex = max(ex, exs[k]);
+  tm.sync();
+  eig_digits(tm, Wout, m, kc, ex, A, nullptr);
+  eig_digits(tm, Qout, n, kc, 0, At, nullptr);
+  *rest = eig_rest(tm, A, At, ex, raw, 1.0 / scale, m, n, kc, reinterpret_cast<double*>(arena));
   tm.sync();
   return 0;
 }

@@ -145,3 +145,43 @@ def test_truncated_factors_are_orthonormal_to_fp64(n, tall, side):
     assert np.abs(d - sg[:k]).max() <= 2.0 ** -52 * np.sqrt(n)     # the tensor itself is rounded as much
     # the inner products of W are those of X times the squares of the singular values (at most 1, at least 0.46)
     assert np.abs(G / np.outer(d, d) - np.eye(k)).max() <= 2.0 ** -51 * np.sqrt(n)
+
+
+def dropped_weight(m, X):
+    """|m - m P|^2 in extended precision, P the projector on the rows of X: an error of X enters squared."""
+    m, X = m.astype(np.longdouble), X.astype(np.longdouble)
+    for _ in range(2):
+        X = 1.5 * X - 0.5 * (X @ X.T) @ X
+    return float(((m - (m @ X.T) @ X) ** 2).sum())
+
+
+@pytest.mark.parametrize("n", [5, 9, 24, 40, 60, 90])
+@pytest.mark.parametrize("low", [0.3, 0.03, 0.011])
+@pytest.mark.parametrize("side", [0, 1])
+def test_a_small_discarded_weight_is_as_accurate_as_a_large_one(n, low, side):
+    """Kept singular values from 1 to 0.5, dropped ones around `low`: down to 2e-4 of the weight is dropped."""
+    rng = np.random.default_rng([n, side])
+    k = max(1, n // 3)
+    sg = np.concatenate([np.linspace(1.0, 0.5, k), low * np.linspace(1.0, 0.5, n - k)])
+    # the isometric factor holds the kept vectors: B for side 0, A for side 1
+    A, B, q = blocks([(n + 3, n) if side == 0 else (n, n + 3)], [sg], rng)
+    An, Bn, kn, disc = gate(A, B, q, side, k, 1e-14)
+    th = np.tensordot(A, B, axes=([2], [0]))
+    assert kn == k
+    if side == 0:
+        ref = dropped_weight(th.reshape(th.shape[0] * 4, -1), Bn.reshape(k, -1))
+    else:
+        ref = dropped_weight(th.reshape(th.shape[0] * 4, -1).T, An.reshape(-1, k).T)
+    # FP64 entries of the remainder, off by 2^-53 of the block's norm (at most sqrt(k)) each, against its norm
+    assert abs(disc - ref) <= 4.0 * 2.0 ** -53 * np.sqrt(k / ref) * ref
+
+
+def test_a_block_that_is_discarded_whole_counts_with_its_norm():
+    rng = np.random.default_rng(1)
+    for n in (5, 24, 40):
+        A, B, q = blocks([(60, 50), (n + 2, n)], [np.linspace(1.0, 0.5, 50), 1e-3 * np.linspace(1.0, 0.5, n)], rng)
+        _, _, k, disc = gate(A, B, q, 0, 50, 1e-14)
+        th = np.tensordot(A[60:], B[:, :, 50:], axes=([2], [0])).astype(np.longdouble)
+        ref = float((th ** 2).sum())
+        # the first block keeps all of its columns
+        assert k == 50 and abs(disc - ref) <= 8.0 * 2.0 ** -53 * ref
