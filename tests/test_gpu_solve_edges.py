@@ -63,3 +63,21 @@ def test_pencils_near_the_ends_of_the_exponent_range(ctx, M, e):
     E, C, r, _ = ctx.solve(H, S)
     E2, C2, r2, _ = ctx.solve(np.ldexp(H, e), S)
     assert r == r2 == M and np.array_equal(np.ldexp(E, e), E2) and np.array_equal(C, C2)
+
+
+@pytest.mark.parametrize("M", [2, 3, 4, 5, 8, 24, 32])
+@pytest.mark.parametrize("span", [0, 4, 10, 22])
+def test_graded_pencils_keep_the_relative_accuracy_of_jacobi(ctx, M, span):
+    """D H D and D S D with D from 1 down to 10^-span: the same energies.  Jacobi's method resolves the small eigenvalues
+    of S relative to themselves (Demmel and Veselic, SIAM J. Matrix Anal. Appl. 13 (1992) 1204)."""
+    for seed in range(3):
+        H, S = pencil(M, seed)
+        L = np.linalg.cholesky(S)
+        ref = np.linalg.eigvalsh(np.linalg.solve(L, np.linalg.solve(L, H).T))
+        D = np.ldexp(1.0, -np.round(span * np.log2(10.0) * np.arange(M) / M).astype(int))   # powers of two: exact
+        E, C, r, _ = ctx.solve_ex(H * D[:, None] * D, S * D[:, None] * D, 0.0)
+        assert r == M
+        # rounding of either route: a few eps of the norms over the smallest eigenvalue of S (1)
+        assert np.abs(E - ref).max() <= 64 * 2.2e-16 * M * np.abs(H).sum(0).max()
+        Cs = C * D[:, None]
+        assert np.abs(Cs.T @ S @ Cs - np.eye(M)).max() <= 64 * 2.2e-16 * M * np.abs(S).sum(0).max()
