@@ -76,14 +76,19 @@ __device__ __forceinline__ float max_nan(float a, float b) {
 }
 // Row stride of the n x n FP32 arrays: a multiple of 4 (16-byte rows) and 4 mod 8, so
 // that 16-byte accesses of eight consecutive rows fall into distinct banks.
-__host__ __device__ __forceinline__ int eig_ld(int n) {
+__host__ __device__ constexpr __forceinline__ int eig_ld(int n) {
   const int l = (n + 3) & ~3;
   return (l & 7) == 4 ? l : l + 4;
 }
-__host__ __device__ __forceinline__ int eig_kp(int k) { return (k + EIG_TC - 1) & ~(EIG_TC - 1); }
+__host__ __device__ constexpr __forceinline__ int eig_kp(int k) { return (k + EIG_TC - 1) & ~(EIG_TC - 1); }
 __host__ __device__ __forceinline__ int pad16(int n) { return (n + 15) & ~15; }
 // floats of the small vectors of eig_start (V: 2 ld, W: ld, P: 2 ld, d, e, tau, lam, scale, a dummy row)
 __host__ __device__ __forceinline__ int eig_vec_floats(int n) { return 11 * eig_ld(n) + 32; }
+// floats that eig_refine needs at least: lk (kp doubles), lh, ek and exs (kp), lam (ld), R (kp x ld), T (n x kp)
+__host__ __device__ constexpr __forceinline__ int eig_refine_words(int n, int kc) {
+  const int kp = eig_kp(kc), ld = eig_ld(n);
+  return 5 * kp + ld + kp * ld + n * kp;
+}
 // Tells the compiler that a generic pointer points to shared memory.
 #define EIG_SHARED(p) __builtin_assume(__isShared(p))
 
@@ -1206,7 +1211,7 @@ __device__ int eig_refine(const Team& tm, uint4* A, uint4* At, int m, int n, int
   // arena: lk (kp doubles), lh, ek and exs (kp), lam (ld), R (kp x ld), then the digits or, after them, T
   // (n x kp) and X (n x ld)
   const int fix = 5 * kp + ld + kp * ld, dig = m16 * kp * EIG_DIG / 2, tx = n * kp;
-  if (fix + tx > words) return 1;
+  if (eig_refine_words(n, kc) > words) return 1;
   double* lk = reinterpret_cast<double*>(arena);
   float* lh = arena + 2 * kp;
   float* ek = lh + kp;

@@ -185,3 +185,37 @@ def test_a_block_that_is_discarded_whole_counts_with_its_norm():
         ref = float((th ** 2).sum())
         # the first block keeps all of its columns
         assert k == 50 and abs(disc - ref) <= 8.0 * 2.0 ** -53 * ref
+
+
+def test_blocks_for_eight_warps_give_the_same_bits_on_every_team():
+    """Blocks of 75 to 104 columns: a pair on a cluster, on one CTA among many, and run again."""
+    w = inputs.make_workload(8, 4, 4, 6, 3, [150, 190, 170], seed=11)
+    with tnqe.Context(w.h1, w.eri, w.N, w.n_alpha, w.n_beta) as g:
+        for m in w.mps:
+            g.add_mps(m.tensors, m.U)
+        base = [(0, 1), (0, 2), (1, 2), (2, 0), (1, 0)]
+        H1, S1 = g.matrix_elements(base)
+        H2, S2 = g.matrix_elements(base * 40)
+        weights = [[g.rotate(i, j) for i, j in base] for _ in range(3)]
+    assert np.array_equal(np.tile(H1, 40), H2) and np.array_equal(np.tile(S1, 40), S2)
+    assert weights[0] == weights[1] == weights[2]
+
+
+@pytest.mark.parametrize("shapes", [[(100, 100)], [(90, 80), (30, 44)], [(52, 52), (60, 74)], [(64, 49), (50, 50)]])
+@pytest.mark.parametrize("keep", [1.0, 0.7])
+def test_wide_blocks_of_which_most_is_kept(shapes, keep):
+    rng = np.random.default_rng(2)
+    A, B, q = blocks(shapes, [np.linspace(1.0 - 0.05 * i, 0.3, min(s)) for i, s in enumerate(shapes)], rng)
+    k = int(keep * sum(min(s) for s in shapes))
+    th = np.tensordot(A, B, axes=([2], [0]))[:, 3, 3, :]
+    sg = np.linalg.svd(th, compute_uv=False)
+    first = None
+    for _ in range(3):
+        An, Bn, kn, disc = gate(A, B, q, 0, k, 1e-14)
+        assert kn == k
+        if first is None:
+            first = An, Bn, disc
+            X = Bn.reshape(k, -1)
+            assert np.abs(X @ X.T - np.eye(k)).max() <= 2.0 ** -51 * np.sqrt(128)
+            assert np.abs(np.sort(np.linalg.norm(An.reshape(-1, k), axis=0))[::-1] - sg[:k]).max() <= 2.0 ** -50 * np.sqrt(128)
+        assert np.array_equal(first[0], An) and np.array_equal(first[1], Bn) and first[2] == disc
