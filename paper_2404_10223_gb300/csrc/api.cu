@@ -8,9 +8,11 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <exception>
 #include <future>
 #include <map>
 #include <memory>
+#include <mutex>
 #include <stdexcept>
 #include <string>
 #include <thread>
@@ -1844,17 +1846,31 @@ void check_ctx(tnqe_ctx* c) {
 // sites 0..N-2), sort every bond by charge and lay the tensors out in that
 // order (host, back to back; offsets in m.off).  Throws Error(TNQE_ERR_ARG).
 // Run f(0..n-1) on up to 8 host threads, the caller's among them (static interleaved shares): one for every
-// 64 K of the `work` entries to visit (about 50 us of a pass; starting a thread costs 20 to 40).
+// 64 K of the `work` entries to visit (about 50 us of a pass; starting a thread costs 20 to 40).  An exception of any
+// share is thrown once all have ended.
 template <class F> void parallel_for(int n, long long work, F f) {
   const int nt = (int)std::max(1LL, std::min({(long long)n, 8LL, (long long)std::thread::hardware_concurrency(),
                                               work / 65536}));
   std::vector<std::thread> th;
-  for (int t = 1; t < nt; ++t)
-    th.emplace_back([&, t]() {
+  th.reserve(nt);
+  std::exception_ptr failed;
+  std::mutex lock;
+  auto share = [&](int t) {
+    try {
       for (int i = t; i < n; i += nt) f(i);
-    });
-  for (int i = 0; i < n; i += nt) f(i);
+    } catch (...) {
+      std::lock_guard<std::mutex> g(lock);
+      if (!failed) failed = std::current_exception();
+    }
+  };
+  try {
+    while ((int)th.size() + 1 < nt) th.emplace_back(share, (int)th.size() + 1);
+  } catch (const std::exception&) {                // no more threads to be had: the caller takes their shares
+  }
+  for (int t = (int)th.size() + 1; t < nt; ++t) share(t);
+  share(0);
   for (auto& x : th) x.join();
+  if (failed) std::rethrow_exception(failed);
 }
 
 // A state's site tensors on the host, sorted by charge, one allocation without
