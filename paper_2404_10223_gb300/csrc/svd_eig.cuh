@@ -250,11 +250,10 @@ __device__ __forceinline__ void mma_tile(const uint4* A, const uint2* D, int it,
         if (i + s + 2 <= NS) mma_bf16(acc[i + s], a[i], b[s]);
   }
 }
-// 2^e, e in [-1022, 1023]
-__device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
-// i as a double, |i| < 2^51 (one FP64 addition; the conversion instruction would be two)
-__device__ __forceinline__ double small_double(long long i) {
-  return __longlong_as_double(0x4338000000000000ll + i) - 6755399441055744.0;
+// i 2^e, |i| < 2^51, |e| < 900 (one FP64 addition; the conversion instruction and the scaling would be three)
+__device__ __forceinline__ double small_double(long long i, int e) {
+  const long long one = 0x4338000000000000ll + ((long long)e << 52);          // 1.5 2^(52 + e)
+  return __longlong_as_double(one + i) - __longlong_as_double(one);
 }
 // The sums of all orders times 2^e, rounded once to FP64: the orders up to 4 and those above as two integers (at
 // most 2^48).
@@ -267,7 +266,7 @@ __device__ __forceinline__ double mma_value(const float (&acc)[NS - 1][4], int q
     if (o < 3) hi = (hi << 8) + x;
     else lo = (lo << 8) + x;
   }
-  return fma(small_double(lo), pow2(e + 4 - 8 * NS), small_double(hi) * pow2(e - 28));
+  return small_double(hi, e - 28) + small_double(lo, e + 4 - 8 * NS);
 }
 
 // ----------------------------------------------------------------------------- Gram matrix
@@ -1136,7 +1135,7 @@ __device__ __noinline__ void eig_update(const Team tm, const float* X, const flo
       for (int q = 0; q < EIG_TC; ++q) {
         const double v = xv[q] + (double)s[q];
         Xd[(size_t)(k0 + q) * ldx + i] = v;
-        if (k0 + q < kc) Xg[(k0 + q) * ld + i] = (float)v;
+        if (k0 + q < kc) Xg[(k0 + q) * ld + i] = X[(k0 + q) * ld + i] + s[q];
       }
     }
   }
