@@ -913,6 +913,13 @@ __device__ int eig_start_at(const Team tm, const uint4* At, int m, int n, float*
     t = warp_sum_f(t);
     if (tr == 0) *trace = t;
   }
+  int coupled = 0;
+  for (int x = tr; x < n * n; x += ts) {
+    const int i = x / n, j = x - i * n;
+    const float g = A[i * ld + j];
+    coupled |= i < j && !(g * g <= 1e-12f * A[i * ld + i] * A[j * ld + j]);
+  }
+  if (!tm.any(coupled)) return 5;
   eig_tridiag(tm, A, n, ld, V, W, P, d, e, tau, inorm + ld);
   const float sc = eig_values(tm, d, e, n, ld, reinterpret_cast<float2*>(P), lam);
   for (int x = tr; x < n * (ld - n); x += ts) X[(x / (ld - n)) * ld + n + x % (ld - n)] = 0.f;
@@ -939,8 +946,8 @@ __device__ int eig_start_at(const Team tm, const uint4* At, int m, int n, float*
 // `words` floats of shared memory (16-byte aligned); Xg (n x ld floats, one vector per
 // row, pad components zero, eigenvalues descending) and lamg (n floats) receive the result, Sg (n x
 // n pairs) and Xalt (n x ld floats, for X where the arena only holds A) are scratch, all
-// in global memory; *trace gets the sum of all eigenvalues.  Returns 0, 1 if the block does not fit (no result), or 3 if X is not
-// orthonormal in the end (the eigenvalues hold).
+// in global memory; *trace gets the sum of all eigenvalues.  Returns 0, 1 if the block does not fit (no result), 3 if X is not
+// orthonormal in the end (the eigenvalues hold), or 5 if the columns of B are orthogonal to FP32 already (no result).
 template <class Team>
 __device__ int eig_start(const Team& tm, const uint4* At, int m, int n, float* arena, int words, float* Xg, float* lamg,
                          float2* Sg, float* Xalt, float* trace) {

@@ -219,3 +219,27 @@ def test_wide_blocks_of_which_most_is_kept(shapes, keep):
             assert np.abs(X @ X.T - np.eye(k)).max() <= 2.0 ** -51 * np.sqrt(128)
             assert np.abs(np.sort(np.linalg.norm(An.reshape(-1, k), axis=0))[::-1] - sg[:k]).max() <= 2.0 ** -50 * np.sqrt(128)
         assert np.array_equal(first[0], An) and np.array_equal(first[1], Bn) and first[2] == disc
+
+
+@pytest.mark.parametrize("n", [1, 2, 8, 9, 24, 60, 90, 120])
+@pytest.mark.parametrize("coupling", [0.0, 1e-13, 1e-8, 1e-5])
+@pytest.mark.parametrize("side", [0, 1])
+def test_columns_that_are_nearly_orthogonal_already(n, coupling, side):
+    """Columns of lengths 0.2 to 1 in mixed order whose inner products are about `coupling`."""
+    rng = np.random.default_rng([n, side])
+    d = rng.permutation(np.linspace(1.0, 0.2, n))
+    M = np.linalg.qr(rng.normal(size=(n + 3, n)))[0] * d
+    M = M @ (np.eye(n) + coupling * rng.normal(size=(n, n)))
+    A, B = np.zeros((n + 3, 4, n)), np.zeros((n, 4, n))
+    A[:, 3], B[:, 3] = M, np.eye(n)
+    keep = max(1, n // 2)
+    An, Bn, k, disc = gate(A, B, ([17] * (n + 3), [34] * n, [51] * n), side, keep, 1e-14)
+    u, sg, vt = np.linalg.svd(M, full_matrices=False)
+    assert k == keep
+    X = Bn.reshape(k, -1) if side == 0 else An.reshape(-1, k).T
+    # the Jacobi SVD: pairs rotated down to m eps
+    assert np.abs(X @ X.T - np.eye(k)).max() <= 4.0 * (n + 3) * 2.0 ** -52
+    new = np.tensordot(An, Bn, axes=([2], [0]))[:, 3, 3, :]
+    gap = 0.8 / max(1, n - 1) if keep < n else 1.0
+    assert np.abs(new - (u[:, :k] * sg[:k]) @ vt[:k]).max() <= 4.0 * (n + 3) * 2.0 ** -52 / gap
+    assert abs(disc - (sg[k:] ** 2).sum()) <= 64 * 2.0 ** -53 * n
