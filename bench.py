@@ -414,7 +414,9 @@ def run_native(args):
                             "hbm": f"hbm_gbs ({peak_src})"}[bound],
             "ms_per_step": t_ms, "work_per_step": work,
             "work_definition": ("rotation: per gate 2 dL dM dR (two-site blocks) + 8 m n (gate) + 4 m n^2 + "
-                                "8 n^3 per m x n charge block (LAPACK-SVD-equivalent), counted in the kernel"
+                                "8 n^3 per m x n charge block (LAPACK-SVD-equivalent), counted in the kernel; most of it "
+                                "runs in FP32 and on the tensor cores, so frac compares with an FP64 LAPACK SVD and does "
+                                "not say how busy the FP64 pipe is"
                                 if top == "rotate_pairs_kernel" else "algorithmic FLOPs of the blocks computed"),
             "breakdown_ms": {k: v[0] for k, v in kern.items()},
             "kernels": {k: {"ms_per_step": v[0], "work_per_step": v[1], "bound": v[2], "unit": v[4],

@@ -35,8 +35,14 @@
 //
 // The products with B run on the tensor cores with operands cut into 8-bit signed
 // digits (Ozaki, Ogita, Oishi, Rump, Numer. Algorithms 59 (2012) 95): every digit is
-// an exact BF16 number, a digit product is at most 2^14 and the sums of one order are
-// integers below 2^24, so FP32 accumulation is exact, and seven digits (resolution
+// an exact BF16 number and a digit product is at most 2^14, so the sum of one order over K
+// entries is an integer of at most (order - 1) K 2^14, exact in FP32 below 2^24: in every
+// order for K <= 146, and for the 256 rows that a bond allows in the orders up to 5 and in
+// all three of the Gram matrix.  Beyond, only digits that are nearly all of one sign and at
+// their limit reach it; then the last unit of such an order is rounded, 2^-44 of the
+// operands' scales in order 6 (whose leading digits would have to be at their limit in both
+// operands, which a unit vector's are not), 2^-52 and 2^-60 in the orders 7 and 8, below the
+// rounding of the result.  Seven digits (resolution
 // 2^-54 of the block's largest entry) with the 28 products of order up to 8 carry the
 // accuracy of FP64 sums.  A multiply-add costs 28/2048
 // of a warp-wide mma against 12 FP32 instructions in double-float and 64 issue cycles
@@ -104,7 +110,9 @@ __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
   return o;
 }
 
-// Uniform in [-1, 1] from a pair of indices (a start vector only has to be generic).
+// Uniform in [-1, 1] from a pair of indices (a start vector only has to be generic): an integer hash, the pair
+// combined by the golden-ratio constant 0x9E3779B1 and 0x85EBCA77 (two primes of Collet's xxHash32), finished with the
+// shifts and multipliers 15, 0x2C1B3C6D, 12, 0x297A2D39, 15 that Wellons found by search (hash-prospector).
 __device__ __forceinline__ float eig_noise(unsigned i, unsigned u) {
   unsigned h = i * 0x9E3779B1u ^ (u + 0x7F4A7C15u) * 0x85EBCA77u;
   h ^= h >> 15;
