@@ -243,3 +243,25 @@ def test_columns_that_are_nearly_orthogonal_already(n, coupling, side):
     gap = 0.8 / max(1, n - 1) if keep < n else 1.0
     assert np.abs(new - (u[:, :k] * sg[:k]) @ vt[:k]).max() <= 4.0 * (n + 3) * 2.0 ** -52 / gap
     assert abs(disc - (sg[k:] ** 2).sum()) <= 64 * 2.0 ** -53 * n
+
+
+@pytest.mark.parametrize("zero", [(), (0,), (1,), (0, 2), (0, 1, 2)])
+@pytest.mark.parametrize("shapes", [[(1, 1), (1, 1), (1, 1)], [(8, 8), (3, 2), (5, 7)], [(40, 8), (1, 8), (2, 30)],
+                                    [(12, 9), (3, 3), (1, 1)]])
+@pytest.mark.parametrize("side", [0, 1])
+def test_gates_of_narrow_blocks_alone_some_of_them_zero(zero, shapes, side):
+    """Blocks of up to 8 columns are done in the first phase (the last set has one of 9); zero blocks have no values."""
+    rng = np.random.default_rng(4)
+    gate(*blocks([(20, 20), (9, 9)], [np.linspace(1.0, 0.1, 20), np.linspace(1.0, 0.1, 9)], rng), side, 9, 0.0)   # other values in the scratch
+    spectra = [np.zeros(min(s)) if b in zero else 1.0 - 0.07 * b - 0.8 * np.arange(min(s)) / min(s) for b, s in enumerate(shapes)]
+    A, B, q = blocks(shapes, spectra, rng)
+    values = np.sort(np.concatenate(spectra))[::-1]
+    keep = max(2, len(values) // 2)
+    An, Bn, k, disc = gate(A, B, q, side, keep, 1e-14)
+    assert k == min(keep, max(1, int((values > 0).sum())))
+    th = np.tensordot(A, B, axes=([2], [0]))[:, 3, 3, :]
+    u, sg, vt = np.linalg.svd(th)
+    got = np.tensordot(An, Bn, axes=([2], [0]))[:, 3, 3, :]
+    # FP64 rounding of sums over up to 40 entries, over gaps of 0.01 and more at the cut
+    assert np.abs(got - (u[:, :k] * sg[:k]) @ vt[:k]).max() <= 2e-13
+    assert abs(disc - (values[k:] ** 2).sum()) <= 1e-14 * len(values)
