@@ -80,8 +80,8 @@ struct RotDesc {
   long long blk_cap;              // doubles of each block buffer below
   long long tile_cap;             // 16 x 16 tiles of the digit fragments
   double* bbuf;                   // SVD blocks B, column-major
-  double* wgbuf;                  // B X (double-floats)
-  double* xdbuf;                  // X (double-floats)
+  double* wgbuf;                  // B X, columns padded to 16
+  double* xdbuf;                  // X, the refined vectors, padded too
   double* dgbuf;                  // digits of either (2 blk_cap)
   uint4* frag;                    // digit fragments of B and B^T (2 x 7 x 32 per tile)
   double* wbuf;                   // B V per block

@@ -31,7 +31,9 @@ namespace {
 // Doubles of staged operand per CTA (24 KiB): nine CTAs of 128 threads share an SM, so that staging, barriers
 // and the ragged ends of the small blocks of some hide behind the FP64 work of the others.  48 KiB (four
 // CTAs): stage 1 of N = 14, chi = 128 23.1 against 19.7 ms, stage 3 17.5 against 14.4; 16 KiB 19.7 and
-// 14.9 (operands in more pieces).
+// 14.9 (operands in more pieces).  At chi = 256, whose items take several pieces: N = 14 stage 1 47.6 ms with 48
+// KiB and 50.0 with 24, stage 3 34.3 and 34.7; N = 20 68.8 and 69, 42.6 and 42.2.  Pieces of stage 3 cut to
+// multiples of the four rows of a thread: 34.6 and 42.3, no difference.
 constexpr int BS_SMEM = 3072;
 
 __device__ __forceinline__ int bs_problem(const long long* prefix, int n, long long x) {
